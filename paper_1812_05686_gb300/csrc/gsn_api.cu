@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/gsn.h.
 #include "../../include/gsn.h"
 #include "gsn_internal.cuh"
+#include "gsn_pair.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -64,6 +65,9 @@ struct gsn_ctx {
     // scratch
     Buf secRq_b, secN_b, secV_b, secW_b, secpart_b, secU_b;  // per-toy buffers of the secondary pieces
     Buf segbuf;              // forward segment prefix [T*G + 1]
+    Buf sppart;              // FP64 in pairs: per-species partial sums
+    Buf pairbuf, batbuf, fbuf, wfbuf, hvybuf;  // FP64 in pairs: column records, batch summaries, centre sums,
+                             // filtered weights, heavy columns
     Buf zerobuf;             // bin-at-zero records [T][G][K][NFZ] (gamma-family responses)
     Buf colbuf, colbuf2, blkbuf, mubuf, wbuf, partbuf, gdirect, devbuf, params, counts_b, win_b, nll_b, grad_b, status_b, Mbuf,
         outbuf;
@@ -168,11 +172,11 @@ int resp_slot(int S, int i) { return i < 5 ? S + i : GSN_SLOT_P(S); }
 // Work decomposition of one launch of T toys.  nsplit: fine-column ranges per forward tile
 // (partial mu rows, summed by the deviance); bw_warps x 32: columns per adjoint block;
 // bw_bsplit: bin ranges per adjoint column block; dev_chunks: deviance blocks per toy.
-Plan plan_with(const gsn_ctx* c, int T, int nsplit, int bw_warps, int bsplit) {
+Plan plan_with(const gsn_ctx* c, int T, int nsplit, int bw_warps, int bsplit, bool pair) {
     Plan p{};
-    const bool e64g = c->opt.precision == GSN_FP64 && c->opt.resolution == GSN_RES_GAUSS;
+    const bool e64g = c->opt.precision == GSN_FP64 && c->opt.resolution == GSN_RES_GAUSS && !pair;
     const int bins_per_tile = 8 * (e64g ? 31 : 32);
-    p.ntile = (c->Jmax + bins_per_tile - 1) / bins_per_tile;
+    p.ntile = (c->Jmax + (pair ? FM : 0) + bins_per_tile - 1) / bins_per_tile;
     p.nsplit = std::max(1, std::min(nsplit, std::max(1, c->K / 256)));
     p.bw_warps = bw_warps;
     p.bw_bsplit = std::max(1, std::min(bsplit, 16));
@@ -184,17 +188,50 @@ Plan plan_with(const gsn_ctx* c, int T, int nsplit, int bw_warps, int bsplit) {
 }
 
 // occupancy heuristic: about 4 blocks per SM in the forward and the adjoint
-Plan heuristic_plan(const gsn_ctx* c, int T) {
+Plan heuristic_plan(const gsn_ctx* c, int T, bool pair) {
     const long long target = 4LL * c->nsm;
-    const Plan p0 = plan_with(c, T, 1, 8, 1);
+    const Plan p0 = plan_with(c, T, 1, 8, 1, pair);
     const long long fw = (long long)T * c->G * p0.ntile;
-    const int nsplit = (int)std::min<long long>((target + fw - 1) / fw, 1 << 20);
+    // in pairs: the tiles of a toy differ in work (band width, quadrature of the low bins), so more and
+    // smaller blocks than fit at once; splits interleave the batches and cost one row of sums each
+    const int nsplit = (int)std::min<long long>(((pair ? 4 : 1) * target + fw - 1) / fw, 1 << 20);
     const long long bw = (long long)T * c->G * p0.nbtask;
     const int bsplit = (int)std::min<long long>((target + bw - 1) / bw, 16);
-    return plan_with(c, T, nsplit, 8, bsplit);
+    return plan_with(c, T, nsplit, 8, bsplit, pair);
 }
 
+Plan heuristic_plan(const gsn_ctx* c, int T) { return heuristic_plan(c, T, c->base.pair != 0); }
+Plan plan_with(const gsn_ctx* c, int T, int nsplit, int bw_warps, int bsplit) {
+    return plan_with(c, T, nsplit, bw_warps, bsplit, c->base.pair != 0);
+}
 Plan make_plan(const gsn_ctx* c, int T) { return heuristic_plan(c, T); }
+
+// sizes of the extra scratch of the FP64 path in pairs, for T toys under plan p: column records,
+// batch summaries, centre sums, filtered weights
+struct PairSizes { size_t rec, bat, f, wf, heavy; };
+PairSizes pair_sizes(const gsn_ctx* c, int T, const Plan& p) {
+    const size_t nb = (size_t)T * c->G * c->base.nbat;
+    return {nb * 32 * sizeof(PairRec), nb * sizeof(float4), (size_t)T * p.nsplit * c->base.fext * sizeof(double),
+            (size_t)T * c->base.fext * sizeof(float2), nb * sizeof(unsigned)};
+}
+void use_pair_buffers(KArgs& a, void* rec, void* bat, void* f, void* wf, void* heavy) {
+    a.pairbuf = (PairRec*)rec; a.batsum = (float4*)bat; a.fbuf = (double*)f; a.wfbuf = (float2*)wf;
+    a.heavy = (unsigned*)heavy;
+}
+
+// ln(1 + u) - u to full relative precision (2 w^3 (1/3 + w^2/5 + ...) - u w, w = u / (2 + u))
+double log1pmx(double u) {
+    if (u < -0.5 || u > 1.0) return std::log1p(u) - u;
+    const double w = u / (2.0 + u), v = w * w;
+    double s = 0.0;
+    for (int n = 22; n >= 1; --n) s = s * v + 1.0 / (2 * n + 1);
+    return 2.0 * w * v * s - u * w;
+}
+void put_pair(std::vector<float>& o, double v) {
+    const float h = (float)v;
+    o.push_back(h);
+    o.push_back((float)(v - (double)h));
+}
 
 void drop_graphs(gsn_ctx* c) {
     for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
@@ -221,6 +258,144 @@ cudaError_t device_ex2_bias(int dev, double& out) {
     }
     out = bias[dev];
     return cudaSuccess;
+}
+
+// Tables of the FP64 response in pairs (gsn_pair64.cu): per 32-bin tile the reference point, per bin
+// centre and per quadrature node the exponent terms (a, D) relative to it, the coefficients of the
+// bin integral over bin centres, 2^(i/1024).
+int pair_tables(gsn_ctx* c, const std::vector<double>& ntab_d, const std::vector<unsigned char>& bcls) {
+    KArgs& a = c->base;
+    Tables& tb = c->tab;
+    const int res = c->opt.resolution;
+    std::vector<double> tref;
+    std::vector<float> snode, qnode;
+    std::vector<unsigned char> qn;
+    std::vector<double> gx, gw;   // Gaussian: eight nodes (six-sigma-wide tails of a sigma of half a bin: 1e-16)
+    gauss_legendre(8, gx, gw);
+    // the exponent terms of a point x of a tile with reference xr
+    auto terms = [&](std::vector<float>& o, double x, double xr) {
+        const double d = x - xr, u = d / xr;
+        put_pair(o, res == GSN_RES_GGAMMA ? std::log1p(u) : d);
+        put_pair(o, res == GSN_RES_GAMMA ? log1pmx(u) : 0.0);
+    };
+    for (int g = 0; g < c->G; ++g) {
+        const std::vector<double>& x = c->edges[tb.g_ds[g][0]];
+        const int J = tb.g_bins[g];
+        // the uniform part: the longest run of equal widths (to rounding) that ends at the last bin
+        const double h0 = x[J] - x[J - 1], xabs = std::max(std::fabs(x[0]), std::fabs(x[J]));
+        int u0 = J - 1;
+        while (u0 > 0 && std::fabs(x[u0 - 1] - (x[J] - (J - u0 + 1) * h0)) <= 64 * 2.3e-16 * xabs) --u0;
+        double h = (x[J] - x[u0]) / (J - u0);
+        for (int j = J; j >= u0; --j)   // against the run's mean width: four roundings of the edges, 1e-12 of a bin
+            if (std::fabs(x[j] - (x[J] - (J - j) * h)) > std::min(4 * 2.3e-16 * xabs, 1e-12 * h)) { u0 = j + 1; h = 0; break; }
+        const int ju = std::max(tb.g_jlin[g], u0 + FM);
+        const bool smooth = h > 0 && ju + 2 * FM <= J;
+        tb.g_ju[g] = smooth ? ju : J;
+        tb.g_h[g] = smooth ? h : 0.0;
+        tb.g_smin[g] = smooth ? (float)(SM_SIGMA * h) : INFINITY;
+        tb.g_tile_off[g] = (int)tref.size() / 4;
+        tb.g_snode_off[g] = (int)snode.size() / 4;
+        const int Jx = J + (smooth ? FM : 0);
+        double hw = 0.0;
+        std::vector<double> xr((Jx + 31) / 32);
+        for (int i = 0; i < (int)xr.size(); ++i) {
+            const int m = 32 * i + 16;
+            xr[i] = m <= J ? x[m] : (smooth ? x[J] + (m - J) * h : x[J]);
+            // ln x_r as a pair (long double: 64 bits or more)
+            const double lx = xr[i] > 0 ? std::log(xr[i]) : 0.0;
+            const double lxl = xr[i] > 0 ? (double)(std::log((long double)xr[i]) - (long double)lx) : 0.0;
+            const double t[4] = {xr[i], lx, xr[i] != 0 ? 1.0 / xr[i] : 0.0, lxl};
+            tref.insert(tref.end(), t, t + 4);
+            if (32 * i < J) hw = std::max({hw, xr[i] - x[32 * i], x[std::min(32 * i + 32, J)] - xr[i]});
+        }
+        double bw = 0.0;
+        for (int j = 0; j < J; ++j) bw = std::max(bw, x[j + 1] - x[j]);
+        tb.g_qmin[g] = (float)(res == GSN_RES_GAUSS ? SQ_GAUSS * bw : SQ_GAMMA * hw);
+        for (int j = 0; j < Jx; ++j) {
+            const double xc = j < J ? 0.5 * (x[j] + x[j + 1]) : x[J] + (j - J + 0.5) * h;
+            terms(snode, xc, xr[j / 32]);
+        }
+        for (int j = 0; j < J; ++j) {
+            const int nb = tb.g_node_off[g] + j;
+            const double* t = ntab_d.data() + (size_t)nb * 3 * NGM_D;
+            const int n = res == GSN_RES_GAUSS ? 8 : bcls[nb] == BIN_ZERO ? 0 : bcls[nb] == BIN_LOG ? NG_LOG_D : NG_LIN_D;
+            qn.push_back((unsigned char)n);
+            for (int i = 0; i < NGM_D; ++i) {
+                if (i >= n) { qnode.insert(qnode.end(), 6, 0.f); continue; }
+                const double hb = 0.5 * (x[j + 1] - x[j]);
+                terms(qnode, res == GSN_RES_GAUSS ? 0.5 * (x[j] + x[j + 1]) + hb * gx[i] : t[i], xr[j / 32]);
+                put_pair(qnode, res == GSN_RES_GAUSS ? hb * gw[i] : t[2 * NGM_D + i]);
+            }
+        }
+    }
+    // (delta / 2) / asinh(delta / 2) in powers of delta^2, as weights of the centres x + m h
+    std::vector<long double> av(FM + 1), bv(FM + 1);
+    std::vector<double> conv(FM + 1, 0.0);
+    auto binom = [](int n, int k) {
+        long double v = 1;
+        for (int i = 1; i <= k; ++i) v = v * (n - k + i) / i;
+        return v;
+    };
+    for (int n = 0; n <= FM; ++n) av[n] = (n & 1 ? -1 : 1) * binom(2 * n, n) / ((2 * n + 1) * std::pow(4.0L, n));
+    for (int n = 0; n <= FM; ++n) {
+        bv[n] = n == 0 ? 1 : 0;
+        for (int k = 1; k <= n; ++k) bv[n] -= av[k] * bv[n - k];
+    }
+    for (int m = 0; m <= FM; ++m) {
+        long double v = 0;
+        for (int n = FM; n >= m; --n) v += bv[n] / std::pow(4.0L, n) * ((n - m) & 1 ? -1 : 1) * binom(2 * n, n - m);
+        conv[m] = (double)v;
+    }
+    std::vector<float> ex;
+    for (int i = 0; i < 1024; ++i) put_pair(ex, std::exp2(i / 1024.0));
+    int rc;
+    const float *p0, *p1;
+    if ((rc = upload(c, ex, &p0))) return rc;
+    a.ex2tab = (const float2*)p0;
+    if ((rc = upload(c, snode, &p1))) return rc;
+    a.snode = (const float4*)p1;
+    if ((rc = upload(c, qnode, &a.qnode))) return rc;
+    if ((rc = upload(c, qn, &a.qn))) return rc;
+    if ((rc = upload(c, tref, &a.tref))) return rc;
+    if ((rc = upload(c, conv, &a.conv))) return rc;
+    // spectra of the per-species kernel, columns outermost
+    bool ok = true;
+    for (double v : c->Sn) ok = ok && (v == 0.0 || v >= SPEC_MIN);
+    if (!ok) return GSN_OK;   // an entry below the range of the pairs: the FP64 kernel
+    const int Spad = (c->S + SPW - 1) / SPW * SPW;
+    std::vector<float> sp((size_t)a.nbat * 32 * Spad * 2, 0.f);
+    std::vector<unsigned> hvy(a.nbat, 0u);   // columns that hold most of a species in their batch: FP64
+    for (int b = 0; b < a.nbat; ++b)
+        for (int s = 0; s < c->S; ++s) {
+            const double* row = &c->Sn[(size_t)s * c->K];
+            const int k1 = std::min(c->K, 32 * b + 32);
+            double tot = 0.0;
+            for (int k = 32 * b; k < k1; ++k) tot += row[k];
+            for (int k = 32 * b; k < k1; ++k)
+                if (row[k] > HEAVY_SHARE * tot) hvy[b] |= 1u << (k & 31);
+        }
+    if ((rc = upload(c, hvy, &a.sp_heavy))) return rc;
+    for (int k = 0; k < c->K; ++k)
+        for (int s = 0; s < c->S && !(hvy[k >> 5] >> (k & 31) & 1); ++s) {
+            const double v = c->Sn[(size_t)s * c->K + k] * SPEC_SCALE;
+            float* o = &sp[((size_t)k * Spad + s) * 2];
+            o[0] = (float)v;
+            o[1] = (float)(v - (double)o[0]);
+        }
+    const float* p2;
+    if ((rc = upload(c, sp, &p2))) return rc;
+    a.Sp = (const float2*)p2;
+    return GSN_OK;
+}
+
+// batch splits and partial sums of the per-species kernel in pairs: about twelve warps per SM
+int reserve_species(gsn_ctx* c, KArgs& a) {
+    if (!a.pair || !a.Sp) return GSN_OK;
+    const long long warps = (long long)a.T * a.G * ((c->Jmax + FM + 31) / 32) * ((a.sp_count + SPW - 1) / SPW);
+    a.sp_nsplit = (int)std::max<long long>(1, std::min<long long>({(12LL * c->nsm + warps - 1) / warps, (a.nbat + 3) / 4, 64}));
+    const int rc = ensure(c, c->sppart, (size_t)a.T * a.G * a.sp_nsplit * c->S * 2 * (c->Jmax + FM) * sizeof(double));
+    a.sp_part = (double*)c->sppart.p;
+    return rc;
 }
 
 int finalize(gsn_ctx* c) {
@@ -430,6 +605,11 @@ int finalize(gsn_ctx* c) {
         a.ft.ds_resp[d] = tb.ds_resp[d];
     }
     int rc;
+    a.pair = (!mixed && c->sec.empty() && a.response) ? 1 : 0;
+    a.fconv = a.pair;
+    a.nbat = (c->K + 31) / 32;
+    a.fext = c->total_bins + c->D * FM;
+    if (a.pair && (rc = pair_tables(c, ntab_d, bcls))) return rc;
     {
         const std::vector<Tables> tv(1, tb);
         if ((rc = upload(c, tv, &a.tb))) return rc;
@@ -538,7 +718,7 @@ int finalize(gsn_ctx* c) {
 }
 
 // allocate (or grow) the scratch buffers for T toys under plan p
-int reserve(gsn_ctx* c, int T, const Plan& p) {
+int reserve(gsn_ctx* c, int T, const Plan& p, bool pair) {
     const size_t rs = c->opt.precision == GSN_MIXED ? sizeof(float) : sizeof(double);
     const int nblk = (c->K + COLBLK - 1) / COLBLK;
     const int npart = NRESP + MAXGDS * c->S;
@@ -556,6 +736,11 @@ int reserve(gsn_ctx* c, int T, const Plan& p) {
     if ((rc = ensure(c, c->gdirect, (size_t)T * c->P * sizeof(double)))) return rc;
     if ((rc = ensure(c, c->devbuf, (size_t)T * p.dev_chunks * (2 + c->base.ntpl) * sizeof(double)))) return rc;
     const KArgs& b = c->base;
+    if (pair) {
+        const PairSizes z = pair_sizes(c, T, p);
+        if ((rc = ensure(c, c->pairbuf, z.rec)) || (rc = ensure(c, c->batbuf, z.bat)) || (rc = ensure(c, c->fbuf, z.f)) ||
+            (rc = ensure(c, c->wfbuf, z.wf)) || (rc = ensure(c, c->hvybuf, z.heavy))) return rc;
+    }
     if (b.nsec) {
         if ((rc = ensure(c, c->secRq_b, (size_t)T * b.Qtot * c->K * rs))) return rc;
         if ((rc = ensure(c, c->secN_b, (size_t)T * b.Qtot * c->S * sizeof(double)))) return rc;
@@ -579,6 +764,7 @@ void fill(gsn_ctx* c, int T, const Plan& p, KArgs& a) {
     a.zerobuf = c->opt.resolution != GSN_RES_GAUSS ? c->zerobuf.p : nullptr;
     a.wbuf = c->wbuf.p; a.partbuf = (double*)c->partbuf.p; a.gdirect = (double*)c->gdirect.p;
     a.devpart = (double*)c->devbuf.p;
+    if (a.pair) use_pair_buffers(a, c->pairbuf.p, c->batbuf.p, c->fbuf.p, c->wfbuf.p, c->hvybuf.p);
     if (a.nsec) {
         a.secRq = c->secRq_b.p;
         a.secN = (double*)c->secN_b.p; a.secV = (double*)c->secV_b.p; a.secW = (double*)c->secW_b.p;
@@ -589,7 +775,7 @@ void fill(gsn_ctx* c, int T, const Plan& p, KArgs& a) {
 
 int prepare(gsn_ctx* c, int T, const Plan& p, KArgs& a) {
     int rc;
-    if ((rc = reserve(c, T, p))) return rc;
+    if ((rc = reserve(c, T, p, a.pair != 0))) return rc;
     fill(c, T, p, a);
     return GSN_OK;
 }
@@ -714,7 +900,8 @@ int choose_plan(gsn_ctx* c, int T, KArgs a, bool grad, Plan& out) {
     const Plan h = heuristic_plan(c, T);
     out = h;
     if (stream_capturing(c)) return GSN_OK;  // no timing inside a caller's capture
-    if (!c->opt.autotune || !c->base.response || (h.nsplit == 1 && h.bw_bsplit == 1)) { c->tuned[key] = h; return GSN_OK; }
+    const bool split = h.bw_bsplit > 1 || (c->base.pair ? (long long)T * c->G * h.ntile < 4LL * c->nsm : h.nsplit > 1);
+    if (!c->opt.autotune || !c->base.response || !split) { c->tuned[key] = h; return GSN_OK; }
     const cudaStream_t st = c->stream;
     int rc;
     if ((rc = prepare(c, T, h, a))) return rc;
@@ -846,7 +1033,7 @@ int batch_device(gsn_ctx* c, int n_toys, const double* params, const double* cou
     }
     // every buffer is sized before any launch is recorded, so a captured graph sees final pointers
     for (size_t i = 0; i < args.size(); ++i)
-        if ((rc = reserve(c, Ts[i], plans[i]))) return rc;
+        if ((rc = reserve(c, Ts[i], plans[i], c->base.pair != 0))) return rc;
     std::vector<long long> key = {1, n_toys, chunk, g ? 1 : 0, (long long)params, (long long)counts, (long long)win,
                                   (long long)nll, (long long)grad, (long long)status};
     for (size_t i = 0; i < args.size(); ++i) {
@@ -930,7 +1117,7 @@ void gsn_destroy(gsn_ctx* c) {
     for (Buf* b : {&c->fit_ws, &c->fit_cfg, &c->fit_eval, &c->fit_ist, &c->wscale_b, &c->rfit_cfg, &c->rfit_ws})
         if (b->p) cudaFree(b->p);
     for (Buf* b : {&c->secRq_b, &c->secN_b, &c->secV_b, &c->secW_b, &c->secpart_b, &c->secU_b,
-                   &c->segbuf, &c->zerobuf, &c->colbuf, &c->colbuf2, &c->blkbuf, &c->mubuf, &c->wbuf, &c->partbuf, &c->gdirect, &c->devbuf, &c->params, &c->counts_b,
+                   &c->sppart, &c->hvybuf, &c->pairbuf, &c->batbuf, &c->fbuf, &c->wfbuf, &c->segbuf, &c->zerobuf, &c->colbuf, &c->colbuf2, &c->blkbuf, &c->mubuf, &c->wbuf, &c->partbuf, &c->gdirect, &c->devbuf, &c->params, &c->counts_b,
                    &c->win_b, &c->nll_b, &c->grad_b, &c->status_b, &c->Mbuf, &c->outbuf, &c->s_hi, &c->s_lo,
                    &c->tc_part, &c->tc_err})
         if (b->p) cudaFree(b->p);
@@ -1311,6 +1498,7 @@ static int compute_species(gsn_ctx* c, const double* params_dev) {
         auto fn = [c](const KArgs& x, cudaStream_t st) { return launch_species_tc(x, c->tm_hi, c->tm_lo, st); };
         if ((rc = launch(c, K_SPECIES, a, fn))) return rc;
     } else {
+        if ((rc = reserve_species(c, a))) return rc;
         if ((rc = launch(c, K_SPECIES, a, launch_species))) return rc;
     }
     return GSN_OK;
@@ -1368,6 +1556,7 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     a.want_grad = 0;
     a.Mbuf = (double*)c->Mbuf.p;  // the cached shapes (one parameter point)
     a.secRq = nullptr;            // the secondary pieces take their slice sums from them
+    a.fconv = 0;                  // mu is complete
     if ((rc = launch(c, K_MU, a, launch_mu_from_species))) return rc;
     if (a.nsec && (rc = launch(c, K_SPECIES, a, launch_secondary))) return rc;
     if ((rc = launch(c, K_DEVIANCE, a, launch_deviance))) return rc;
@@ -1577,7 +1766,12 @@ int gsn_fit_rates_batch_dev(gsn_ctx* c, int n_toys, double* params_dev, const do
     for (int t0 = 0; t0 < n_toys; t0 += chunk) {
         const int T = std::min(chunk, n_toys - t0);
         KArgs a = c->base;
-        const Plan p = make_plan(c, T);
+        // The Newton iteration's Hessian is FP32 and its weak directions amplify the last bits of the
+        // shapes: the path and the iteration count of a toy are those of these very bits, so the FP64
+        // shapes keep the FP64 kernel (in pairs they agree to 1e-14, and three fits in four then took
+        // another number of iterations to the same minimum)
+        a.pair = 0;
+        const Plan p = heuristic_plan(c, T, false);
         if ((rc = prepare(c, T, p, a))) return rc;
         a.params = params_dev + (size_t)t0 * P; a.params_stride = P;
         a.counts = toy_counts_dev + (size_t)t0 * c->n_counts; a.counts_stride = c->n_counts;
@@ -1730,21 +1924,31 @@ extern "C" int gsn_eval_grad_noalloc(gsn_ctx* c, const double* params_dev, doubl
     unsigned char* base = static_cast<unsigned char*>(noalloc_address(c->dev, err));
     if (!base) return fail(c, GSN_ERR_CUDA, err);
     KArgs a = c->base;
-    const Plan p = make_plan(c, 1);
     const size_t rs = c->opt.precision == GSN_MIXED ? sizeof(float) : sizeof(double);
-    const size_t sizes[10] = {
-        (size_t)c->G * c->K * NFP * rs,                         // column records
-        (size_t)c->G * a.nblk * 2 * rs,                         // band summaries
-        (size_t)p.nsplit * c->total_bins * sizeof(double),      // partial mu
-        (size_t)c->total_bins * rs,                             // w
-        (size_t)c->G * p.nbtask * a.NPART * sizeof(double),     // partial gradients
-        (size_t)c->P * sizeof(double),                          // direct gradient terms
-        (size_t)p.dev_chunks * (2 + c->base.ntpl) * sizeof(double),   // deviance and template partials
-        c->opt.resolution == GSN_RES_GGAMMA ? (size_t)c->G * c->K * NFG * sizeof(double) : 0,  // adjoint coefficients
-        ((size_t)c->G + 1) * sizeof(int),                       // forward segment prefix
-        c->opt.resolution != GSN_RES_GAUSS ? (size_t)c->G * c->K * NFZ * rs : 0};  // bin-at-zero records
-    size_t off[10], total = 0;
-    for (int i = 0; i < 10; ++i) { off[i] = total; total += (sizes[i] + 255) & ~(size_t)255; }
+    constexpr int NBUF = 15;
+    Plan p;
+    size_t off[NBUF], total;
+    // FP64 in pairs where its records fit the array, else the FP64 kernels, which need less
+    for (int pair = a.pair;; pair = 0) {
+        a.pair = a.fconv = pair;
+        p = heuristic_plan(c, 1, pair != 0);
+        const PairSizes z = pair ? pair_sizes(c, 1, p) : PairSizes{0, 0, 0, 0, 0};
+        const size_t sizes[NBUF] = {
+            (size_t)c->G * c->K * NFP * rs,                         // column records
+            (size_t)c->G * a.nblk * 2 * rs,                         // band summaries
+            (size_t)p.nsplit * c->total_bins * sizeof(double),      // partial mu
+            (size_t)c->total_bins * rs,                             // w
+            (size_t)c->G * p.nbtask * a.NPART * sizeof(double),     // partial gradients
+            (size_t)c->P * sizeof(double),                          // direct gradient terms
+            (size_t)p.dev_chunks * (2 + c->base.ntpl) * sizeof(double),   // deviance and template partials
+            c->opt.resolution == GSN_RES_GGAMMA ? (size_t)c->G * c->K * NFG * sizeof(double) : 0,  // adjoint coefficients
+            ((size_t)c->G + 1) * sizeof(int),                       // forward segment prefix
+            c->opt.resolution != GSN_RES_GAUSS ? (size_t)c->G * c->K * NFZ * rs : 0,  // bin-at-zero records
+            z.rec, z.bat, z.f, z.wf, z.heavy};
+        total = 0;
+        for (int i = 0; i < NBUF; ++i) { off[i] = total; total += (sizes[i] + 255) & ~(size_t)255; }
+        if (!pair || total <= GSN_NOALLOC_SCRATCH_BYTES) break;
+    }
     if (total > GSN_NOALLOC_SCRATCH_BYTES)
         return fail(c, GSN_ERR_ARG, "this problem needs " + std::to_string(total) + " bytes of scratch; the "
                     "no-allocation entry point holds " + std::to_string((size_t)GSN_NOALLOC_SCRATCH_BYTES));
@@ -1756,6 +1960,7 @@ extern "C" int gsn_eval_grad_noalloc(gsn_ctx* c, const double* params_dev, doubl
     a.dev_chunks = p.dev_chunks; a.devpart = (double*)(base + off[6]);
     a.colbuf2 = (double*)(base + off[7]);
     a.segoff = (int*)(base + off[8]);
+    if (a.pair) use_pair_buffers(a, base + off[10], base + off[11], base + off[12], base + off[13], base + off[14]);
     a.zerobuf = c->opt.resolution != GSN_RES_GAUSS ? (void*)(base + off[9]) : nullptr;
     a.params = params_dev; a.params_stride = c->P;
     a.counts_stride = 0; a.win_stride = 0;

@@ -181,11 +181,11 @@ DEV void gg_inc_gamma(double a, double y, double& P, double& Pa, double& py) {
 // Column prologue of the generalized gamma (FP64 for both precisions).  Fills the record fields
 // that depend on the response (everything but TN), the band [xmin, xmax] and the adjoint record
 // g (NFG values); mu, var: the column's mean and variance, p the power, deq = d E_q / d kB.
-// Returns the normalisation N_k that multiplies the T_dk (mixed: the density at the mean times
+// lfmu, kappa1, Amu: ln f(mu), kappa_1 and (mu/s)^p.  Returns the normalisation N_k that multiplies the T_dk (mixed: the density at the mean times
 // ex2_scale = 1 / (1 + b), b the SFU exponentials' measured mean relative error; FP64: 1).
 template <class R>
 DEV double gg_column(double mu, double var, double p, double cut, double x1, bool zero_bin, bool mixed,
-                     double ex2_scale, R* f, R* z, double* gco, R& xmin, R& xmax) {
+                     double ex2_scale, R* f, R* z, double* gco, R& xmin, R& xmax, double& lfmu, double& kappa1, double& Amu) {
     const double a = 1.0 / p;
     const double r = log1p(var / (mu * mu));
     double Hx, lxs;                                   // dH/dx at the root, ln(d/p)
@@ -198,6 +198,7 @@ DEV double gg_column(double mu, double var, double p, double cut, double x1, boo
     const double k1 = (d - 1.0) - p * A;
     // density at the mean: ln f(mu) = ln p - ln mu + d ln(mu/s) - A - lnGamma(d/p)
     const double lfm = log(p) - log(mu) + d * ls - A - lgx;
+    lfmu = lfm; kappa1 = k1; Amu = A;
     double Nk = 1.0;
     if (mixed) {
         Nk = exp(lfm) * ex2_scale;

@@ -73,6 +73,12 @@ struct Tables {
     int g_active[MAXG];         // some dataset of the group has smeared species
     double g_rscale[MAXG][NRESP];  // fixed multipliers of the response parameters (section 2.4 slices)
     int sp_kind[MAXS];
+    // FP64 response in FP32 pairs (gsn_pair64.cu)
+    int g_ju[MAXG];             // first bin that smooth columns integrate over bin centres (the bin count: none)
+    int g_tile_off[MAXG];       // the group's 32-bin tiles in tref
+    int g_snode_off[MAXG];      // its bin centres in snode
+    double g_h[MAXG];           // bin width of the uniform part
+    float g_smin[MAXG], g_qmin[MAXG];  // smallest sigma of a smooth batch, of a batch evaluated in pairs
 };
 
 // Copy of the first FASTG groups and FASTD datasets of Tables, carried in the kernel parameters
@@ -86,6 +92,8 @@ struct FastTables {
     int ds_off[FASTD], ds_bins[FASTD], ds_group[FASTD], ds_resp[FASTD];
     int sp_kind[MAXS];          // complete (the species count is at most MAXS)
 };
+
+struct PairRec;
 
 struct KArgs {
     // problem
@@ -188,6 +196,25 @@ struct KArgs {
     void* secRq;           // [T][Qtot][K] of Real: N_k sum_{j in q} R_jk (NULL: slice sums from Mbuf)
     // statistics: evaluated (bin, column) pairs per kernel class (NULL = off)
     unsigned long long* work;
+    // FP64 response in FP32 pairs (gsn_pair64.cu): tables, per-launch records and sums
+    int pair;                   // the context's response kernels work in pairs
+    int fconv;                  // the deviance adds the smooth columns' bin integrals from fbuf
+    const float2* ex2tab;       // [1024] 2^(i/1024)
+    const double* conv;         // [FM + 1] coefficients of the bin integral over bin centres
+    const double* tref;         // [tile][4] reference point x_r, ln x_r, 1/x_r
+    const float4* snode;        // [node] (a, D) of the bin centres, FM of them above the histogram
+    const float* qnode;         // [bin][NGM_D][6] (a, D, weight) of the quadrature nodes
+    const unsigned char* qn;    // [bin] quadrature nodes of the bin (0: the bin at zero)
+    int nbat, fext;             // batches of 32 columns; total_bins + D FM
+    PairRec* pairbuf;           // [T][G][nbat 32]
+    float4* batsum;             // [T][G][nbat] band, smallest sigma, smallest sigma of smooth columns
+    unsigned* heavy;            // [T][G][nbat] columns evaluated in FP64 (bit per column of the batch)
+    const unsigned* sp_heavy;   // [nbat] the same for the per-species sums
+    double* fbuf;               // [T][nsplit][fext] sum_k T_k f_k at the bin centres
+    float2* wfbuf;              // [T][fext] filtered weights
+    const float2* Sp;           // [nbat 32][S padded to SPW] S' SPEC_SCALE (NULL: spectra the pairs do not hold)
+    int sp_nsplit;              // batch splits of the per-species kernel
+    double* sp_part;            // [T][G][sp_nsplit][S][centres, bins][Jmax + FM]
     // tensor-core per-species contraction
     int tc_nsplit;         // column ranges per bin tile
     double* tc_part;       // [tc_nsplit][G][S][Jmax] partial sums
@@ -257,6 +284,9 @@ cudaError_t launch_deviance(const KArgs& a, cudaStream_t st);
 cudaError_t launch_devfinal(const KArgs& a, cudaStream_t st);
 cudaError_t launch_backward(const KArgs& a, cudaStream_t st);
 cudaError_t launch_gradfinal(const KArgs& a, cudaStream_t st);
+cudaError_t launch_forward_pair(const KArgs& a, cudaStream_t st);
+cudaError_t launch_backward_pair(const KArgs& a, cudaStream_t st);
+cudaError_t launch_species_pair(const KArgs& a, cudaStream_t st);
 cudaError_t launch_species(const KArgs& a, cudaStream_t st);
 cudaError_t launch_mu_from_species(const KArgs& a, cudaStream_t st);
 cudaError_t launch_expected_out(const KArgs& a, cudaStream_t st);

@@ -21,8 +21,44 @@
 // deviance and reductions.  FP64: everything in double.
 #include "gsn_device.cuh"
 #include "gsn_ggamma.cuh"
+#include "gsn_pair.cuh"
 
 namespace gsn {
+
+// Band of a gamma column of shape d, x = mu (1 + t): conservative bounds lo, hi of the t where
+// h(t) = (d-1) D(t) - t exceeds -c (lo = -1: down to 0)
+template <class R> DEV void gamma_band(R c, R d, R& lo, R& hi) {
+    R thi;
+    if (d >= R(1)) {
+        const R bq = R(2) - R(2) * c;
+        thi = (-bq + sqrt(bq * bq + R(8) * c * (d + R(1)))) / (R(2) * (d + R(1)));
+    } else {
+        thi = c / d;
+    }
+    // for d > 1, h + cut is concave: Newton steps from these outer bounds stay outside the band
+    if (d > R(1)) {
+        for (int it = 0; it < 3; ++it) {
+            const R L1 = log1p(thi);
+            const R h = (d - R(1)) * (L1 - thi) - thi + c;
+            const R hp = -(d - R(1)) * thi / (R(1) + thi) - R(1);
+            thi = thi - h / hp;
+        }
+    }
+    hi = thi;
+    lo = R(-1);
+    if (d > R(1)) {
+        R tlo = -(R(1) + sqrt(R(1) + R(2) * c * (d - R(1)))) / (d - R(1));
+        if (tlo > R(-1)) {
+            for (int it = 0; it < 3; ++it) {
+                const R L1 = log1p(tlo);
+                const R h = (d - R(1)) * (L1 - tlo) - tlo + c;
+                const R hp = -(d - R(1)) * tlo / (R(1) + tlo) - R(1);
+                tlo = fmax(tlo - h / hp, tlo);
+            }
+            lo = tlo;
+        }
+    }
+}
 
 // ------------------------------------------------------------- columns -----
 template <class R, int RES, bool FAST>
@@ -70,6 +106,11 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
     __syncthreads();
 
     R xmin = (R)INFINITY, xmax = (R)-INFINITY;
+    [[maybe_unused]] double psig = INFINITY, psmooth = INFINITY;  // sigma; sigma if smooth (0 if not)
+    // FP64 gamma family: ln f(mu), ln mu as a pair, ln d - psi(d); generalized gamma: kappa_1, (mu/s)^p
+    [[maybe_unused]] double pfm = 0.0, plm = 0.0, pkc = 0.0, pk1 = 0.0, pAp = 0.0;
+    [[maybe_unused]] float plml = 0.f;
+    [[maybe_unused]] float pT = 0.f;   // largest |T| of the column over the group's datasets
     if (k < a.K) {
         R* rec = colrec<R>(a, t, g, k);
         R f[NFP], z[NFZ];
@@ -89,6 +130,7 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
             }
             const double mud = LY * Eq;
             const double vard = fma(mud, fma(rc, mud, rb), ra);
+            psig = sqrt(vard);
             const double D = L - y, r1 = y / (1.0 + y);
             f[F_DEQ] = (R)(beta > 0 ? (a.s0 * (beta / alpha) * (2.0 * D + y * r1) - a.s1 * (D + y * r1)) / (alpha * alpha) : NAN);
             f[F_MUH] = (R)mud;
@@ -96,7 +138,8 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
             double gco[NFG];
             const double x1 = a.edges[tb_g_edge_off<FAST>(a, g) + 1];
             Nk = (R)gg_column<R>(mud, vard, sres[5], a.cut, x1, tb_g_zero<FAST>(a, g) != 0, sizeof(R) == 4, a.ex2_scale, f, z, gco,
-                                 xmin, xmax);
+                                 xmin, xmax, pfm, pk1, pAp);
+            if constexpr (sizeof(R) == 8) plm = log(mud);
             double* g2 = a.colbuf2 + (((long long)t * a.G + g) * a.K + k) * NFG;
 #pragma unroll
             for (int i = 0; i < NFG; ++i) g2[i] = gco[i];
@@ -140,6 +183,7 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
             }
             // in FP64 and rounded once: FP32 copies of a, b, c would scale every column's variance alike
             var = (R)fma((double)mu, fma(rc, (double)mu, rb), ra);
+            if constexpr (sizeof(R) == 8) psig = sqrt(var);
             f[F_DEQ] = deq;
             if constexpr (RES == 0) {
                 const R sig = sqrt(var), isg = R(1) / sig;
@@ -195,42 +239,56 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
                         f[F_KAPPA] = (float)(log(dd) - digamma_d(dd));
                     }
                 } else {
-                    f[F_A] = -d * log(s) - lgamma(d);
+                    if (a.pair) {
+                        // ln mu to ~1e-17 from the logarithm of the nearest tile's reference point (a pair
+                        // made on the host) and log1p of the small rest: the exponent takes (d - 1) ln(x / mu),
+                        // d ~ 1000, and a rounding of ln mu would shift the whole column by 4e-13
+                        {
+                            const double* tr = a.tref + 4LL * a.tb->g_tile_off[g];
+                            int lo = 0, hi = (tb_g_bins<FAST>(a, g) + 31) / 32 - 1;   // last reference <= mu (or the first)
+                            while (lo < hi) { const int m = (lo + hi + 1) >> 1; if (tr[4 * m] <= mu) lo = m; else hi = m - 1; }
+                            const double xr = tr[4 * lo], u = (mu - xr) / xr;
+                            if (fabs(u) < 0.5) {
+                                const double l1 = log1p(u), hi1 = tr[4 * lo + 1] + l1, b = hi1 - tr[4 * lo + 1];
+                                plml = (float)((tr[4 * lo + 1] - (hi1 - b)) + (l1 - b) + tr[4 * lo + 3]);
+                                plm = hi1;
+                            } else {
+                                plm = log(mu);
+                            }
+                        }
+                        if (d >= GG_XSTIR) {
+                            // Stirling: ln f(mu) = -ln(2 pi var) / 2 - tail(d), ln d - psi(d) = 1/(2d) - tail'(d)
+                            double lt, dt, id;
+                            gg_tails(d, lt, dt, id);
+                            pfm = -0.5 * log(6.283185307179586477 * var) - lt;
+                            pkc = 0.5 * id - dt;
+                            f[F_A] = fma(-(d - 1.0), plm, pfm + d);
+                        } else {
+                            const double ls = log(s), A = -d * ls - lgamma(d);
+                            pfm = fma(d - 1.0, plm, A - d);
+                            pkc = log(d) - digamma_d(d);
+                            f[F_A] = A;
+                        }
+                        f[F_KAPPA] = plm - pkc;   // ln s + psi(d), s d = mu
+                    } else {
+                        f[F_A] = -d * log(s) - lgamma(d);
+                        f[F_KAPPA] = log(s) + digamma_d(d);
+                    }
                     f[F_B] = d - 1.0;
                     f[F_C] = 1.0 / s;
-                    f[F_KAPPA] = log(s) + digamma_d(d);
                 }
-                // conservative band from bounds on h(t) = (d-1) D(t) - t, x = mu (1 + t)
-                const R c = (R)a.cut;
-                R thi;
-                if (d >= R(1)) {
-                    const R bq = R(2) - R(2) * c;
-                    thi = (-bq + sqrt(bq * bq + R(8) * c * (d + R(1)))) / (R(2) * (d + R(1)));
+                // FP32 bounds in pairs too: they need only be conservative, and six FP64 logarithms per
+                // column cost as much as the rest of it; the cut is widened by 0.01 against their rounding
+                if (sizeof(R) == 8 && a.pair) {
+                    float lo, hi;
+                    gamma_band<float>((float)a.cut + 0.01f, (float)d, lo, hi);
+                    xmax = mu * (R(1) + (R)hi);
+                    xmin = lo > -1.0f ? mu * (R(1) + (R)lo) : R(0);
                 } else {
-                    thi = c / d;
-                }
-                // for d > 1, h + cut is concave: Newton steps from these outer bounds stay outside the band
-                if (d > R(1)) {
-                    for (int it = 0; it < 3; ++it) {
-                        const R L1 = log1p(thi);
-                        const R h = (d - R(1)) * (L1 - thi) - thi + c;
-                        const R hp = -(d - R(1)) * thi / (R(1) + thi) - R(1);
-                        thi = thi - h / hp;
-                    }
-                }
-                xmax = mu * (R(1) + thi);
-                xmin = 0;
-                if (d > R(1)) {
-                    R tlo = -(R(1) + sqrt(R(1) + R(2) * c * (d - R(1)))) / (d - R(1));
-                    if (tlo > R(-1)) {
-                        for (int it = 0; it < 3; ++it) {
-                            const R L1 = log1p(tlo);
-                            const R h = (d - R(1)) * (L1 - tlo) - tlo + c;
-                            const R hp = -(d - R(1)) * tlo / (R(1) + tlo) - R(1);
-                            tlo = fmax(tlo - h / hp, tlo);
-                        }
-                        xmin = mu * (R(1) + tlo);
-                    }
+                    R lo, hi;
+                    gamma_band<R>((R)a.cut, d, lo, hi);
+                    xmax = mu * (R(1) + hi);
+                    xmin = lo > R(-1) ? mu * (R(1) + lo) : R(0);
                 }
                 if (tb_g_zero<FAST>(a, g)) {
                     const R x1 = (R)a.edges[tb_g_edge_off<FAST>(a, g) + 1];
@@ -275,6 +333,43 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
                 f[F_TN0 + dd] = T * Nk;
             }
         }
+        if constexpr (sizeof(R) == 8) {
+            if (a.pair) {
+                constexpr double L2 = 1.4426950408889634074;
+                PairRec pr{};
+                double Nn = 1.0, P = 0.0, shape = SM_SHAPE;
+                if constexpr (RES == 0) {
+                    pr.A = f[F_MUH]; pr.B = f[F_A];
+                    P = -0.5 * L2 * f[F_A] * f[F_A];
+                    Nn = f[F_A] * INV_SQRT2PI;
+                } else {
+                    const double ms = f[F_MUH] / psig;
+                    pr.mu = f[F_MUH];
+                    pr.A = pfm; pr.lmh = plm; pr.lml = plml;
+                    if constexpr (RES == 1) {
+                        pr.B = f[F_B]; pr.C = f[F_C];
+                        P = L2 * f[F_B];
+                        pr.kc.x = (float)pkc; pr.kc.y = (float)(pkc - (double)pr.kc.x);
+                    } else {
+                        pr.B = pk1; pr.C = pAp;
+                    }
+                    shape = fmin(f[F_B] + 1.0, ms * ms);
+                }
+                pr.Ph = (float)P; pr.Pl = (float)(P - (double)pr.Ph);
+                bool ok = isfinite(f[F_XMIN]) && isfinite(f[F_XMAX]) && isfinite(pr.A) && isfinite(P) && fabs(P) < 1e12;
+                for (int dd = 0; dd < MAXGDS; ++dd) {
+                    const double T = dd < tb_g_nds<FAST>(a, g) ? f[F_TN0 + dd] * Nn : 0.0;
+                    pr.T[dd].x = (float)T; pr.T[dd].y = (float)(T - (double)pr.T[dd].x);
+                    pT = fmaxf(pT, fabsf(pr.T[dd].x));
+                    ok = ok && (T == 0.0 || (fabs(T) > PAIR_TMIN && fabs(T) < PAIR_TMAX));
+                }
+                a.pairbuf[((long long)t * a.G + g) * a.nbat * 32 + k] = pr;
+                // a column that the pairs do not take sends its batch to the FP64 formulas
+                if (!ok || !(psig > 0.0)) psig = 0.0;
+                psmooth = psig > 0.0 && shape >= SM_SHAPE ? psig : 0.0;
+                if (!(isfinite(f[F_XMIN]) && isfinite(f[F_XMAX]))) { xmin = (R)-INFINITY; xmax = (R)INFINITY; }
+            }
+        }
 #pragma unroll
         for (int i = 0; i < NFP; ++i) rec[i] = f[i];
         if (a.zerobuf) {
@@ -285,6 +380,21 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
     }
     // band summary of this column block
     R mn = warp_min<R>(xmin), mx = warp_max<R>(xmax);
+    if constexpr (sizeof(R) == 8) {
+        if (a.pair) {
+            const int b = k >> 5;
+            const double s0 = warp_min<double>(psig), s1 = warp_min<double>(psmooth);
+            if (k >= a.K && b < a.nbat) a.pairbuf[((long long)t * a.G + g) * a.nbat * 32 + k] = PairRec{};
+            // columns that outweigh their batch (mono-energetic lines): the sums would take over the
+            // single error of their pairs, 6e-15, which elsewhere averages out over the columns
+            const float tot = warp_sum<float>(pT);
+            const unsigned heavy = __ballot_sync(0xffffffffu, pT > HEAVY_SHARE * tot && psig > 0.0);
+            if ((threadIdx.x & 31) == 0 && b < a.nbat) a.heavy[((long long)t * a.G + g) * a.nbat + b] = heavy;
+            if ((threadIdx.x & 31) == 0 && b < a.nbat)  // band bounds rounded outwards
+                a.batsum[((long long)t * a.G + g) * a.nbat + b] =
+                    make_float4(__double2float_rd(mn), __double2float_ru(mx), __double2float_rd(s0), __double2float_rd(s1));
+        }
+    }
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0) { sred[0][w] = mn; sred[1][w] = mx; }
     __syncthreads();
@@ -531,6 +641,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
     const int t = blockIdx.x, c = blockIdx.y;
     __shared__ double sh[32];
     __shared__ PeakInfo pk;
+    __shared__ double fs[sizeof(R) == 8 ? 256 + 2 * FM : 1];
     __shared__ double tcoef[MAXS];    // eps_d f_ds r_s of the dataset's Monte Carlo templates
     __shared__ long long toff[MAXS];  // and the offsets of their histograms
     const double* prm = a.params + (long long)t * a.params_stride;
@@ -564,10 +675,44 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
             __syncthreads();
         }
         const double* ed = a.edges + tb_g_edge_off(a, tb_ds_group(a, d));
-        for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+        // smooth columns (FP64 in pairs): the sums at the bin centres of a strip of bins, with FM on
+        // either side, from which every bin takes its integral; 0 where no column reaches the centre
+        [[maybe_unused]] const double* frow = nullptr;
+        [[maybe_unused]] int ju = J, flo = 0, fhi = 0;
+        if constexpr (sizeof(R) == 8) {
+            if (a.fconv && tb_ds_resp(a, d) && a.tb->g_ju[tb_ds_group(a, d)] < J) {
+                int ulo, uhi;
+                toy_window_union(a, t, tb_ds_group(a, d), ulo, uhi);
+                ju = a.tb->g_ju[tb_ds_group(a, d)];
+                if (uhi > ju) { flo = max(ulo, ju) - FM; fhi = uhi + FM; }
+                frow = a.fbuf + (long long)t * a.nsplit * a.fext + off + d * FM;
+            }
+        }
+        for (int s0 = j0; s0 < j1; s0 += blockDim.x) {
+            const int j = s0 + threadIdx.x;
+            if constexpr (sizeof(R) == 8) {
+                if (fhi > flo) {
+                    __syncthreads();  // earlier readers of fs are done
+                    for (int i = threadIdx.x; i < (int)blockDim.x + 2 * FM; i += blockDim.x) {
+                        const int n = s0 - FM + i;
+                        fs[i] = n >= flo && n < fhi ? sum_splits(frow + n, a.fext, a.nsplit) : 0.0;
+                    }
+                    __syncthreads();
+                }
+            }
+            if (j >= j1) continue;
             double w = 0.0;
             if (j >= lo && j < hi) {
                 double mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nsplit) : 0.0;
+                if constexpr (sizeof(R) == 8) {
+                    const double* f = fs + threadIdx.x + FM;
+                    if (fhi > flo && j >= ju && f[0] != 0.0) {
+                        double v = 0.0;
+#pragma unroll
+                        for (int m = FM; m > 0; --m) v = fma(a.conv[m], f[-m] + f[m], v);
+                        mu = fma(fma(a.conv[0], f[0], v), ed[j + 1] - ed[j], mu);
+                    }
+                }
                 for (int q = 0; q < npk; ++q) {
                     if (j < pk.lo[q] || j >= pk.hi[q]) continue;
                     const double m = pk.m[q], wd = pk.w[q];
@@ -1382,6 +1527,7 @@ cudaError_t launch_columns(const KArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_forward(const KArgs& a, cudaStream_t st) {
+    if (a.pair) return launch_forward_pair(a, st);
     dim3 grid(a.ntile, a.nsplit, a.T * a.G);
     if (a.precision == 1) {
         // the generalized gamma of free power runs the general per-node kernel
@@ -1408,6 +1554,7 @@ cudaError_t launch_devfinal(const KArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_backward(const KArgs& a, cudaStream_t st) {
+    if (a.pair) return launch_backward_pair(a, st);
     // the tuned mixed adjoint serves the Gaussian and gamma responses (with or without secondary observables)
     if (a.precision == 1 && a.res != 2) return launch_backward_mixed(a, st);
     dim3 grid(a.nbtask, a.G, a.T);
@@ -1429,6 +1576,7 @@ cudaError_t launch_gradfinal(const KArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_species(const KArgs& a, cudaStream_t st) {
+    if (a.pair && a.Sp) return launch_species_pair(a, st);
     const int nchunk = (a.sp_count + 15) / 16;
     if (a.precision == 0 && a.res == 0) {
         dim3 grid((a.Jmax + FWD_WARPS * 31 - 1) / (FWD_WARPS * 31), a.G, nchunk * a.T);
