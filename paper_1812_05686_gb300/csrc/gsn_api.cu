@@ -31,6 +31,8 @@ struct gsn_ctx {
     Buf rfit_cfg, rfit_ws;   // gsn_fit_rates_batch_dev: bounds and indices; design rows, mu
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    cudaStream_t aux = nullptr;                       // work forked from and joined to the stream within a step
+    cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     int nsm = 1;
     std::string err;
     // problem, host copies
@@ -851,6 +853,17 @@ int run_step(gsn_ctx* c, KArgs& a, bool grad) {
         if ((rc = launch(c, K_FORWARD, a, launch_forward))) return rc;
     }
     if ((rc = launch(c, K_DEVIANCE, a, launch_deviance))) return rc;
+    if (grad && a.response && !c->prof) {
+        // the NLL's final sum and the peaks' gradient (one block per toy) run beside the adjoint; both
+        // read the deviance's results and gradfinal waits for both
+        CUDA_TRY(c, cudaEventRecord(c->fork_ev, c->stream));
+        CUDA_TRY(c, cudaStreamWaitEvent(c->aux, c->fork_ev, 0));
+        CUDA_TRY(c, launch_devfinal(a, c->aux));
+        CUDA_TRY(c, cudaEventRecord(c->join_ev, c->aux));
+        if ((rc = launch(c, K_BACKWARD, a, launch_backward))) return rc;
+        CUDA_TRY(c, cudaStreamWaitEvent(c->stream, c->join_ev, 0));
+        return launch(c, K_GRADFINAL, a, launch_gradfinal);
+    }
     if ((rc = launch(c, K_DEVFINAL, a, launch_devfinal))) return rc;
     if (grad) {
         if (a.response && (rc = launch(c, K_BACKWARD, a, launch_backward))) return rc;
@@ -1096,6 +1109,13 @@ int gsn_create(gsn_ctx** out, const gsn_options* opt) {
         if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return GSN_ERR_CUDA; }
         c->own_stream = true;
     }
+    if (cudaStreamCreateWithFlags(&c->aux, cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming) != cudaSuccess) {
+        cudaGetLastError();
+        gsn_destroy(c);
+        return GSN_ERR_CUDA;
+    }
     cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->dev);
     if (c->nsm <= 0) c->nsm = 1;
     if (o.precision == GSN_MIXED && device_ex2_bias(c->dev, c->ex2_bias) != cudaSuccess) {
@@ -1124,6 +1144,9 @@ void gsn_destroy(gsn_ctx* c) {
     if (c->work.p) cudaFree(c->work.p);
     for (auto& p : c->pending) { c->event_pool.push_back(p.e0); c->event_pool.push_back(p.e1); }
     for (cudaEvent_t e : c->event_pool) cudaEventDestroy(e);
+    if (c->aux) { cudaStreamSynchronize(c->aux); cudaStreamDestroy(c->aux); }
+    if (c->fork_ev) cudaEventDestroy(c->fork_ev);
+    if (c->join_ev) cudaEventDestroy(c->join_ev);
     if (c->own_stream) cudaStreamDestroy(c->stream);
     delete c;
 }

@@ -621,10 +621,18 @@ DEV int load_peaks(const KArgs& a, const double* prm, int d, PeakInfo& pk) {
     return pk.n;
 }
 
-// sum of the nsplit partial mu rows of one bin, in a fixed order (four interleaved accumulators)
+// sum of the nsplit partial mu rows of one bin, in a fixed order; eight loads in flight (a single
+// point has ~80 rows per bin, and one block per 128 bins)
 DEV double sum_splits(const double* p, long long stride, int n) {
     double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
     int i = 0;
+    for (; i + 8 <= n; i += 8) {
+        double v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = p[(i + q) * stride];
+        s0 += v[0]; s1 += v[1]; s2 += v[2]; s3 += v[3];
+        s0 += v[4]; s1 += v[5]; s2 += v[6]; s3 += v[7];
+    }
     for (; i + 4 <= n; i += 4) {
         s0 += p[i * stride]; s1 += p[(i + 1) * stride];
         s2 += p[(i + 2) * stride]; s3 += p[(i + 3) * stride];
@@ -1190,45 +1198,69 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_b
 }
 
 // ------------------------------------------------------------ gradfinal ----
-__global__ void __launch_bounds__(128) k_gradfinal(KArgs a) {
+// One block per toy, group by group (fixed order): the tasks' partials of every value are summed by
+// several threads, each a fixed share of the tasks with its loads independent (a single point has
+// hundreds of tasks and one thread per value walked them one dependent load after another), then
+// every parameter gathers the values of the slots it fills, in slot order.
+constexpr int GF_THREADS = 512;
+__global__ void __launch_bounds__(GF_THREADS) k_gradfinal(KArgs a) {
     const int t = blockIdx.x;
-    __shared__ double vals[NRESP + MAXGDS * MAXS];  // one group's reduced partials
+    __shared__ double vals[GF_THREADS];              // shares, then one group's reduced partials
+    __shared__ double gslot[MAXGDS * MAXS];          // rate gradients of the group's datasets
+    __shared__ int pslot[MAXGDS * MAXS];             // and their parameters (-1: none)
     double* gr = a.grad + (long long)t * a.P;
-    if (threadIdx.x == 0) {
-        const double* gd = a.gdirect + (long long)t * a.P;
-        for (int p = 0; p < a.P; ++p) gr[p] = gd[p];
-    }
-    // group by group (fixed order): sum of the per-task partials, then the slot-map scatter
+    const double* gd = a.gdirect + (long long)t * a.P;
+    for (int p = threadIdx.x; p < a.P; p += GF_THREADS) gr[p] = gd[p];
+    const int nv = a.NPART, shares = max(1, GF_THREADS / nv);
+    const int v = threadIdx.x % nv, sh = threadIdx.x / nv;
     for (int g = 0; g < a.G; ++g) {
         if (!tb_g_active(a, g)) continue;  // no adjoint partials for groups without smeared species
-        for (int v = threadIdx.x; v < a.NPART; v += blockDim.x) {
-            const double* p = a.partbuf + ((long long)t * a.G + g) * a.nbtask * a.NPART + v;
-            double s = 0.0;
-            for (int task = 0; task < a.nbtask; ++task) s += p[(long long)task * a.NPART];
-            vals[v] = s;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            // the slots hold unscaled parameters: d(scale p)/dp = scale
-            for (int i = 0; i < NRESP; ++i)
-                if (tb_g_resp(a, g, i) >= 0) gr[tb_g_resp(a, g, i)] += vals[i] * tb_g_rscale(a, g, i);
-            for (int dd = 0; dd < tb_g_nds(a, g); ++dd) {
-                const int d = tb_g_ds(a, g, dd);
-                for (int s = 0; s < a.S; ++s) {
-                    const double f = a.rfac[d * a.S + s];
-                    if (a.ft.sp_kind[s] >= 2 || f == 0.0) continue;
-                    const int p = a.slot_map[d * a.NSLOT + s];
-                    if (p >= 0) gr[p] += f * vals[NRESP + dd * a.S + s];
-                }
+        const double* row = a.partbuf + ((long long)t * a.G + g) * a.nbtask * nv;
+        double s = 0.0;
+        if (sh < shares) {
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+            int task = sh;
+            for (; task + 3 * shares < a.nbtask; task += 4 * shares) {
+                s0 += row[(long long)task * nv + v];
+                s1 += row[(long long)(task + shares) * nv + v];
+                s2 += row[(long long)(task + 2 * shares) * nv + v];
+                s3 += row[(long long)(task + 3 * shares) * nv + v];
             }
+            for (; task < a.nbtask; task += shares) s0 += row[(long long)task * nv + v];
+            s = (s0 + s1) + (s2 + s3);
+        }
+        __syncthreads();  // the previous group's readers are done
+        vals[threadIdx.x] = s;
+        const int nds = tb_g_nds(a, g);
+        for (int i = threadIdx.x; i < nds * a.S; i += GF_THREADS) {
+            const int d = tb_g_ds(a, g, i / a.S), sp = i % a.S;
+            const bool smeared = a.ft.sp_kind[sp] < 2 && a.rfac[d * a.S + sp] != 0.0;
+            pslot[i] = smeared ? a.slot_map[d * a.NSLOT + sp] : -1;
+            gslot[i] = a.rfac[d * a.S + sp];
         }
         __syncthreads();
+        if (threadIdx.x < nv) {
+            double r = 0.0;
+            for (int q = 0; q < shares; ++q) r += vals[q * nv + threadIdx.x];
+            if (threadIdx.x >= NRESP && threadIdx.x < NRESP + nds * a.S) gslot[threadIdx.x - NRESP] *= r;
+            s = r;   // the response values stay with the threads below NRESP
+        }
+        __syncthreads();
+        if (threadIdx.x < NRESP) vals[threadIdx.x] = s;
+        __syncthreads();
+        // the slots hold unscaled parameters: d(scale p)/dp = scale
+        for (int p = threadIdx.x; p < a.P; p += GF_THREADS) {
+            double r = gr[p];
+            for (int i = 0; i < NRESP; ++i)
+                if (tb_g_resp(a, g, i) == p) r += vals[i] * tb_g_rscale(a, g, i);
+            for (int i = 0; i < nds * a.S; ++i)
+                if (pslot[i] == p) r += gslot[i];
+            gr[p] = r;
+        }
     }
-    if (threadIdx.x == 0) {
-        bool fin = true;
-        for (int p = 0; p < a.P; ++p) fin = fin && isfinite(gr[p]);
-        if (!fin && a.status && a.status[t] == 0) a.status[t] = -4;
-    }
+    bool bad = false;
+    for (int p = threadIdx.x; p < a.P; p += GF_THREADS) bad = bad || !isfinite(gr[p]);
+    if (__syncthreads_or(bad) && threadIdx.x == 0 && a.status && a.status[t] == 0) a.status[t] = -4;
 }
 
 // ---------------------------------------------------- per-species path -----
@@ -1571,7 +1603,7 @@ cudaError_t launch_backward(const KArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_gradfinal(const KArgs& a, cudaStream_t st) {
-    k_gradfinal<<<a.T, 128, 0, st>>>(a);
+    k_gradfinal<<<a.T, GF_THREADS, 0, st>>>(a);
     return cudaGetLastError();
 }
 
