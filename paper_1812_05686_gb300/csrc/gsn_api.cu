@@ -75,7 +75,7 @@ struct gsn_ctx {
         outbuf;
     unsigned long long scratch_gen = 0;  // bumped whenever a buffer is (re)allocated
     // launch plans chosen by the autotuner, per (toys in a launch, gradient wanted)
-    struct PlanRec { int nsplit, ntile, bw_warps, bw_bsplit, nbtask, dev_chunks; };
+    struct PlanRec { int nsplit, nsub, ntile, bw_warps, bw_bsplit, nbtask, dev_chunks; };
     std::map<std::pair<int, int>, PlanRec> tuned;
     // CUDA graphs of recent launch sequences, replayed when the same sequence repeats
     struct GraphRec { std::vector<long long> key; cudaGraphExec_t exec; };
@@ -180,6 +180,13 @@ Plan plan_with(const gsn_ctx* c, int T, int nsplit, int bw_warps, int bsplit, bo
     const int bins_per_tile = 8 * (e64g ? 31 : 32);
     p.ntile = (c->Jmax + (pair ? FM : 0) + bins_per_tile - 1) / bins_per_tile;
     p.nsplit = std::max(1, std::min(nsplit, std::max(1, c->K / 256)));
+    // shares of a split's batches for the two-bin mixed forward: from four waves of its warps (24 per
+    // SM) down, the last wave is a large part of the launch; a share costs one more row of mu to add
+    p.nsub = 1;
+    if (c->opt.precision == GSN_MIXED && c->opt.resolution == GSN_RES_GAMMA && (long long)T * c->G >= 32) {
+        const long long warps = (long long)T * c->G * ((c->Jmax + 63) / 64) * p.nsplit;
+        p.nsub = (int)std::max<long long>(1, std::min<long long>(8, 4 * 24LL * c->nsm / warps));
+    }
     p.bw_warps = bw_warps;
     p.bw_bsplit = std::max(1, std::min(bsplit, 16));
     const int ncb = (c->K + p.bw_warps * 32 - 1) / (p.bw_warps * 32);
@@ -592,6 +599,7 @@ int finalize(gsn_ctx* c) {
         noff += J;
     }
     a.Jmax = c->Jmax;
+    for (int g = 0; g < c->G; ++g) a.jlin_max = std::max(a.jlin_max, tb.g_jlin[g]);
     // kernel-parameter copy of the first groups and datasets
     a.fast = (c->G <= FASTG && c->D <= FASTD) ? 1 : 0;
     for (int g = 0; g < std::min(c->G, FASTG); ++g) {
@@ -732,7 +740,7 @@ int reserve(gsn_ctx* c, int T, const Plan& p, bool pair) {
         (rc = ensure(c, c->colbuf2, (size_t)T * c->G * c->K * NFG * sizeof(double)))) return rc;
     if ((rc = ensure(c, c->blkbuf, (size_t)T * c->G * nblk * 2 * rs))) return rc;
     if ((rc = ensure(c, c->segbuf, ((size_t)T * c->G + 1) * sizeof(int)))) return rc;
-    if ((rc = ensure(c, c->mubuf, (size_t)T * p.nsplit * c->total_bins * sizeof(double)))) return rc;
+    if ((rc = ensure(c, c->mubuf, (size_t)T * p.nsplit * p.nsub * c->total_bins * sizeof(double)))) return rc;
     if ((rc = ensure(c, c->wbuf, (size_t)T * c->total_bins * rs))) return rc;
     if ((rc = ensure(c, c->partbuf, (size_t)T * c->G * p.nbtask * npart * sizeof(double)))) return rc;
     if ((rc = ensure(c, c->gdirect, (size_t)T * c->P * sizeof(double)))) return rc;
@@ -758,7 +766,7 @@ int reserve(gsn_ctx* c, int T, const Plan& p, bool pair) {
 void fill(gsn_ctx* c, int T, const Plan& p, KArgs& a) {
     a.work = nullptr;
     a.T = T;
-    a.nsplit = p.nsplit; a.ntile = p.ntile;
+    a.nsplit = p.nsplit; a.nsub = p.nsub; a.nrow = p.nsplit * p.nsub; a.ntile = p.ntile;
     a.bw_warps = p.bw_warps; a.bw_bsplit = p.bw_bsplit; a.nbtask = p.nbtask;
     a.dev_chunks = p.dev_chunks;
     a.colbuf = c->colbuf.p; a.colbuf2 = (double*)c->colbuf2.p; a.blkbuf = c->blkbuf.p; a.mubuf = (double*)c->mubuf.p;
@@ -1570,7 +1578,7 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     if ((rc = species_cached(c, params, hit))) return rc;
     KArgs a = c->base;
     Plan p = make_plan(c, 1);
-    p.nsplit = 1;
+    p.nsplit = p.nsub = 1;
     if ((rc = prepare(c, 1, p, a))) return rc;
     a.params = (const double*)c->params.p; a.params_stride = c->P;
     a.counts_stride = 0; a.win_stride = 0;
@@ -1955,11 +1963,12 @@ extern "C" int gsn_eval_grad_noalloc(gsn_ctx* c, const double* params_dev, doubl
     for (int pair = a.pair;; pair = 0) {
         a.pair = a.fconv = pair;
         p = heuristic_plan(c, 1, pair != 0);
+        p.nsub = 1;
         const PairSizes z = pair ? pair_sizes(c, 1, p) : PairSizes{0, 0, 0, 0, 0};
         const size_t sizes[NBUF] = {
             (size_t)c->G * c->K * NFP * rs,                         // column records
             (size_t)c->G * a.nblk * 2 * rs,                         // band summaries
-            (size_t)p.nsplit * c->total_bins * sizeof(double),      // partial mu
+            (size_t)p.nsplit * p.nsub * c->total_bins * sizeof(double),  // partial mu
             (size_t)c->total_bins * rs,                             // w
             (size_t)c->G * p.nbtask * a.NPART * sizeof(double),     // partial gradients
             (size_t)c->P * sizeof(double),                          // direct gradient terms
@@ -1976,7 +1985,7 @@ extern "C" int gsn_eval_grad_noalloc(gsn_ctx* c, const double* params_dev, doubl
         return fail(c, GSN_ERR_ARG, "this problem needs " + std::to_string(total) + " bytes of scratch; the "
                     "no-allocation entry point holds " + std::to_string((size_t)GSN_NOALLOC_SCRATCH_BYTES));
     a.T = 1;
-    a.nsplit = p.nsplit; a.ntile = p.ntile;
+    a.nsplit = p.nsplit; a.nsub = p.nsub; a.nrow = p.nsplit * p.nsub; a.ntile = p.ntile;
     a.bw_warps = p.bw_warps; a.bw_bsplit = p.bw_bsplit; a.nbtask = p.nbtask;
     a.colbuf = base + off[0]; a.blkbuf = base + off[1]; a.mubuf = (double*)(base + off[2]);
     a.wbuf = base + off[3]; a.partbuf = (double*)(base + off[4]); a.gdirect = (double*)(base + off[5]);

@@ -146,13 +146,15 @@ struct KArgs {
     void* zerobuf;         // [T][G][K][NFZ] of Real: bin-at-zero values (gamma-family responses)
     double* colbuf2;       // [T][G][K][NFG]: adjoint coefficients (generalized gamma only)
     void* blkbuf;          // [T][G][nblk][2] of Real: min xmin, max xmax
-    double* mubuf;         // [T][nsplit][total_bins]
+    double* mubuf;         // [T][nrow][total_bins]
     void* wbuf;            // [T][total_bins] of Real
     double* partbuf;       // [T][G][nbtask][NPART]
     double* gdirect;       // [T][P]
     int nblk;
     int nbtask, bw_warps, bw_bsplit, NPART;
     int ntile;             // forward tiles per group (max over groups)
+    int nsub, nrow;        // shares of a split's column batches (mixed forward); rows of mubuf, nsplit nsub
+    int jlin_max;          // largest g_jlin
     int* segoff;           // [T*G + 1] gamma forward: exclusive prefix of the 64-bin segments of every
                            // (toy, group) window (written by the forward launcher)
     int dev_chunks;        // deviance blocks per toy

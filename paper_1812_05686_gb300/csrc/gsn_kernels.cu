@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
     const int chunk = (a.total_bins + a.dev_chunks - 1) / a.dev_chunks;
     const int b0 = c * chunk, b1 = min(a.total_bins, b0 + chunk);
     const long long sstride = a.total_bins;
-    const double* mrow = a.mubuf + (long long)t * a.nsplit * a.total_bins;
+    const double* mrow = a.mubuf + (long long)t * a.nrow * a.total_bins;
     double part = 0.0;
     int bad_mu = 0, bad_fin = 0;
     for (int d = 0; d < a.D; ++d) {
@@ -711,7 +711,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
             if (j >= j1) continue;
             double w = 0.0;
             if (j >= lo && j < hi) {
-                double mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nsplit) : 0.0;
+                double mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
                 if constexpr (sizeof(R) == 8) {
                     const double* f = fs + threadIdx.x + FM;
                     if (fhi > flo && j >= ju && f[0] != 0.0) {
@@ -1203,8 +1203,42 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_b
 // hundreds of tasks and one thread per value walked them one dependent load after another), then
 // every parameter gathers the values of the slots it fills, in slot order.
 constexpr int GF_THREADS = 512;
+
+// sum of a (toy, group)'s task partials of value v over every shares-th task from sh
+DEV double task_share(const double* row, int nv, int v, int sh, int shares, int ntask) {
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int task = sh;
+    for (; task + 3 * shares < ntask; task += 4 * shares) {
+        s0 += row[(long long)task * nv + v];
+        s1 += row[(long long)(task + shares) * nv + v];
+        s2 += row[(long long)(task + 2 * shares) * nv + v];
+        s3 += row[(long long)(task + 3 * shares) * nv + v];
+    }
+    for (; task < ntask; task += shares) s0 += row[(long long)task * nv + v];
+    return (s0 + s1) + (s2 + s3);
+}
+
+// Problems of many response groups (GF_GROUPS or more): the partials of every (toy, group) are summed
+// by a block of their own into the group's first task row, and k_gradfinal reads that row only (one
+// block walking 64 groups one after another took 20 us per group)
+constexpr int GF_GROUPS = 4;
+__global__ void __launch_bounds__(GF_THREADS) k_gradsum(KArgs a) {
+    const int t = blockIdx.x, g = blockIdx.y;
+    if (!tb_g_active(a, g)) return;
+    __shared__ double vals[GF_THREADS];
+    const int nv = a.NPART, shares = max(1, GF_THREADS / nv), v = threadIdx.x % nv, sh = threadIdx.x / nv;
+    double* row = a.partbuf + ((long long)t * a.G + g) * a.nbtask * nv;
+    vals[threadIdx.x] = sh < shares ? task_share(row, nv, v, sh, shares, a.nbtask) : 0.0;
+    __syncthreads();
+    if (threadIdx.x < nv) {
+        double r = 0.0;
+        for (int q = 0; q < shares; ++q) r += vals[q * nv + threadIdx.x];
+        row[threadIdx.x] = r;
+    }
+}
+
 __global__ void __launch_bounds__(GF_THREADS) k_gradfinal(KArgs a) {
-    const int t = blockIdx.x;
+    const int t = blockIdx.x, ntask = a.G >= GF_GROUPS ? 1 : a.nbtask;
     __shared__ double vals[GF_THREADS];              // shares, then one group's reduced partials
     __shared__ double gslot[MAXGDS * MAXS];          // rate gradients of the group's datasets
     __shared__ int pslot[MAXGDS * MAXS];             // and their parameters (-1: none)
@@ -1216,19 +1250,7 @@ __global__ void __launch_bounds__(GF_THREADS) k_gradfinal(KArgs a) {
     for (int g = 0; g < a.G; ++g) {
         if (!tb_g_active(a, g)) continue;  // no adjoint partials for groups without smeared species
         const double* row = a.partbuf + ((long long)t * a.G + g) * a.nbtask * nv;
-        double s = 0.0;
-        if (sh < shares) {
-            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-            int task = sh;
-            for (; task + 3 * shares < a.nbtask; task += 4 * shares) {
-                s0 += row[(long long)task * nv + v];
-                s1 += row[(long long)(task + shares) * nv + v];
-                s2 += row[(long long)(task + 2 * shares) * nv + v];
-                s3 += row[(long long)(task + 3 * shares) * nv + v];
-            }
-            for (; task < a.nbtask; task += shares) s0 += row[(long long)task * nv + v];
-            s = (s0 + s1) + (s2 + s3);
-        }
+        double s = sh < shares ? task_share(row, nv, v, sh, shares, ntask) : 0.0;
         __syncthreads();  // the previous group's readers are done
         vals[threadIdx.x] = s;
         const int nds = tb_g_nds(a, g);
@@ -1603,6 +1625,7 @@ cudaError_t launch_backward(const KArgs& a, cudaStream_t st) {
 }
 
 cudaError_t launch_gradfinal(const KArgs& a, cudaStream_t st) {
+    if (a.G >= GF_GROUPS && a.response) k_gradsum<<<dim3(a.T, a.G), GF_THREADS, 0, st>>>(a);
     k_gradfinal<<<a.T, GF_THREADS, 0, st>>>(a);
     return cudaGetLastError();
 }

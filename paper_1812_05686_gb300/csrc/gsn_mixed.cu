@@ -122,42 +122,61 @@ DEV float pair_value(const RecF& c, float xc, float dl, float lp, float lm, floa
 }
 
 // ------------------------------------------------------------- forward -----
-template <int RES, int NDS, bool FAST>
-__global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_m(KArgs a) {
-    const int tile = blockIdx.x, split = blockIdx.y;
-    const int t = blockIdx.z / a.G, g = blockIdx.z % a.G;
-    if (!tb_g_active<FAST>(a, g)) return;  // no smeared species in the group
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __shared__ RecF srec[FWD_WARPS][32];
-    int wlo, whi;
-    toy_window_union<FAST>(a, t, g, wlo, whi);
-    // warps tile the toy's window from its first bin, so no warp starts outside it
-    const int j0 = wlo + (tile * FWD_WARPS + warp) * 32;
-    if (j0 >= whi) return;
-    const int j = j0 + lane;
-    const bool valid = j < whi;
-    const int jr = min(j, whi - 1);
-    const int nb = tb_g_node_off<FAST>(a, g) + jr;
-    const int jf = j0, jl = min(j0 + 31, whi - 1);
-    const float xlo_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + jf];
-    const float xhi_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + jl + 1];
-    const int nds = tb_g_nds<FAST>(a, g);
-    const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
-    const int k_beg = split * kchunk, k_end = min(a.K, k_beg + kchunk);
+// column range of a window segment's band within columns [k_beg, k_end): first and last 256-column
+// block that overlaps
+DEV void band_columns(const KArgs& a, int t, int g, int k_beg, int k_end, float xlo_w, float xhi_w, int& kfirst, int& klast) {
     const float* blk = reinterpret_cast<const float*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
-
-    // column range of the band: first and last 256-column block that overlaps
-    int kfirst = k_end, klast = k_beg;
+    kfirst = k_end; klast = k_beg;
     for (int b = k_beg / COLBLK; b * COLBLK < k_end; ++b) {
         if (blk[2 * b + 1] < xlo_w || blk[2 * b] > xhi_w) continue;
         kfirst = min(kfirst, max(b * COLBLK, k_beg));
         klast = max(klast, min((b + 1) * COLBLK, k_end));
     }
+}
+// the sub-th share of the batches of 32 columns in [kfirst, klast): the batches, and so their FP32 sums,
+// are those of the whole range
+DEV void share_batches(int sub, int nsub, int& kfirst, int& klast) {
+    const int nb = (klast - kfirst + 31) / 32, per = (nb + nsub - 1) / nsub;
+    const int k0 = kfirst + 32 * per * sub;
+    klast = min(klast, k0 + 32 * per);
+    kfirst = k0;
+}
 
-    double accd[MAXGDS] = {};
+// Segments with bins below the first linear bin (log-spaced nodes, the bin at zero) take the general
+// node table for all their bins.  They are few (the first one or two of a window) and every column of
+// the lowest ~100 p.e. reaches them, so one warp walking those columns from global memory was the
+// longest chain of a launch: a whole block takes the segment, its warps every eighth batch of 32
+// columns from shared memory, and the warps' sums are added in a fixed order.  With the batches of a
+// split shared among several warps where a launch has few (nsub), the forward of 4 toys x 64 response
+// groups takes 7.8 ms (18.3), of one two-dataset point 66 us (158), of 4096 toys 24.5 ms (28.2: the
+// general path also cost the others registers).
+struct LowRec { float4 r[4]; };
+
+template <int RES, int HALVES>
+__global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_low(KArgs a) {
+    __shared__ LowRec srec_all[FWD_WARPS * 32];
+    __shared__ double sred[FWD_WARPS * 32];
+    const int t = blockIdx.z / a.G, g = blockIdx.z % a.G, row0 = blockIdx.y * a.nsub;
+    if (!tb_g_active(a, g)) return;
+    int wlo, whi;
+    toy_window_union(a, t, g, wlo, whi);
+    const int j0 = wlo + blockIdx.x * 32 * HALVES;   // segments tile the window from its first bin
+    if (j0 >= whi || j0 >= tb_g_jlin(a, g)) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    LowRec* srec = srec_all + warp * 32;
+    const int nds = tb_g_nds(a, g), jl = min(j0 + 32 * HALVES - 1, whi - 1);
+    const float xlo_w = (float)a.edges[tb_g_edge_off(a, g) + j0];
+    const float xhi_w = (float)a.edges[tb_g_edge_off(a, g) + jl + 1];
+    const int kchunk = (a.K + a.nsplit - 1) / a.nsplit, k_beg = blockIdx.y * kchunk;
+    int kfirst, klast;
+    band_columns(a, t, g, k_beg, min(a.K, k_beg + kchunk), xlo_w, xhi_w, kfirst, klast);
+    const float4* rec = reinterpret_cast<const float4*>(colrec<float>(a, t, g, 0));
     int ncol = 0;
-    if (j0 < tb_g_jlin<FAST>(a, g)) {  // the warp holds bins below the first linear bin
-        // warp holds bins of the general node table (log-spaced or the bin at zero)
+#pragma unroll 1
+    for (int h = 0; h < HALVES; ++h) {
+        const int j = j0 + 32 * h + lane;
+        const bool valid = j < whi;
+        const int nb = tb_g_node_off(a, g) + min(j, whi - 1);
         const unsigned char cls = a.bclass[nb];
         const float* nodes = a.ntab_f + (long long)nb * 3 * NGM_F;
         const float xc = a.xc_f[nb];
@@ -166,17 +185,83 @@ __global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_m(KArgs a) {
         for (int n = 0; n < NG_LOG_F; ++n) {
             del[n] = nodes[n]; lam[n] = nodes[NGM_F + n]; wt[n] = valid ? nodes[2 * NGM_F + n] : 0.f;
         }
-        for (int k = kfirst; k < klast; ++k) {
-            const float* c = colrec<float>(a, t, g, k);
-            if (c[F_XMAX] < xlo_w || c[F_XMIN] > xhi_w) continue;
-            ++ncol;
-            float v = bin_value_f<RES, NG_LOG_F>(c, xc, del, lam, wt);
-            if (RES == 1 && cls == BIN_ZERO) v = valid ? zerorec<float>(a, t, g, k)[Z_P0] : 0.0f;
+        double accd[MAXGDS] = {};
+        ncol = 0;
+        for (int kb = kfirst + warp * 32; kb < klast; kb += 32 * FWD_WARPS) {
+            const int k = kb + lane;
+            LowRec q;
+            q.r[2] = make_float4(INFINITY, -INFINITY, 0.f, 0.f);   // (XMIN, XMAX, T0, T1)
+            if (k < klast) {
 #pragma unroll
-            for (int dd = 0; dd < MAXGDS; ++dd)
-                if (dd < nds) accd[dd] += (double)(v * c[F_TN0 + dd]);
+                for (int i = 0; i < 4; ++i) q.r[i] = rec[(long long)k * 4 + i];
+            }
+            unsigned m = __ballot_sync(0xffffffffu, !(q.r[2].y < xlo_w || q.r[2].x > xhi_w));
+            __syncwarp();
+            srec[lane] = q;
+            __syncwarp();
+            ncol += __popc(m);
+            float s[MAXGDS] = {}, cc[MAXGDS] = {};
+            while (m) {
+                const int ci = __ffs(m) - 1;
+                m &= m - 1;
+                const float* c = reinterpret_cast<const float*>(&srec[ci]);
+                float v = bin_value_f<RES, NG_LOG_F>(c, xc, del, lam, wt);
+                if (RES == 1 && cls == BIN_ZERO) v = valid ? zerorec<float>(a, t, g, kb + ci)[Z_P0] : 0.0f;
+#pragma unroll
+                for (int dd = 0; dd < MAXGDS; ++dd)
+                    if (dd < nds) two_sum_acc(s[dd], cc[dd], __fmul_rn(v, c[F_TN0 + dd]));
+            }
+#pragma unroll
+            for (int dd = 0; dd < MAXGDS; ++dd) accd[dd] += (double)s[dd] + (double)cc[dd];
         }
-    } else {
+        for (int dd = 0; dd < nds; ++dd) {
+            __syncthreads();
+            sred[warp * 32 + lane] = accd[dd];
+            __syncthreads();
+            if (warp == 0 && valid) {
+                double v = 0.0;
+                for (int w = 0; w < FWD_WARPS; ++w) v += sred[w * 32 + lane];
+                double* out = a.mubuf + ((long long)t * a.nrow + row0) * a.total_bins + tb_ds_off(a, tb_g_ds(a, g, dd)) + j;
+                out[0] = v;
+                for (int r = 1; r < a.nsub; ++r) out[(long long)r * a.total_bins] = 0.0;
+            }
+        }
+    }
+    if (a.work) {
+        if (lane == 0) atomicAdd(&a.work[K_FORWARD], (unsigned long long)ncol * (unsigned long long)(jl - j0 + 1));
+    }
+}
+
+template <int RES, int NDS, bool FAST>
+__global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_m(KArgs a) {
+    const int split = blockIdx.y;
+    const int t = blockIdx.z / a.G, g = blockIdx.z % a.G;
+    if (!tb_g_active<FAST>(a, g)) return;  // no smeared species in the group
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ RecF srec[FWD_WARPS][32];
+    int wlo, whi;
+    toy_window_union<FAST>(a, t, g, wlo, whi);
+    const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
+    const int k_beg = split / a.nsub * kchunk, k_end = min(a.K, k_beg + kchunk);
+    const int tile = blockIdx.x;
+    // warps tile the toy's window from its first bin, so no warp starts outside it
+    const int j0 = wlo + (tile * FWD_WARPS + warp) * 32;
+    if (j0 >= whi || j0 < tb_g_jlin<FAST>(a, g)) return;  // (below: k_forward_low)
+    const int j = j0 + lane;
+    const bool valid = j < whi;
+    const int jr = min(j, whi - 1);
+    const int nb = tb_g_node_off<FAST>(a, g) + jr;
+    const int jf = j0, jl = min(j0 + 31, whi - 1);
+    const float xlo_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + jf];
+    const float xhi_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + jl + 1];
+    const int nds = tb_g_nds<FAST>(a, g);
+    int kfirst, klast;
+    band_columns(a, t, g, k_beg, k_end, xlo_w, xhi_w, kfirst, klast);
+    share_batches(split % a.nsub, a.nsub, kfirst, klast);
+
+    double accd[MAXGDS] = {};
+    int ncol = 0;
+    {
         const float4 b0 = reinterpret_cast<const float4*>(a.btab_f)[2 * nb];
         const float4 b1 = reinterpret_cast<const float4*>(a.btab_f)[2 * nb + 1];
         const float xc = b0.x, dl = b0.y, lp = b0.z, lm = b0.w;
@@ -245,7 +330,7 @@ __global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_m(KArgs a) {
         if (lane == 0) atomicAdd(&a.work[K_FORWARD], (unsigned long long)ncol * __popc(m));
     }
     if (valid) {
-        double* out = a.mubuf + ((long long)t * a.nsplit + split) * a.total_bins;
+        double* out = a.mubuf + ((long long)t * a.nrow + split) * a.total_bins;
 #pragma unroll
         for (int dd = 0; dd < MAXGDS; ++dd)
             if (dd < nds) out[tb_ds_off<FAST>(a, tb_g_ds<FAST>(a, g, dd)) + j] = accd[dd];
@@ -342,9 +427,13 @@ template <int NDS, bool FAST>
 __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m2(KArgs a) {
     const int split = blockIdx.y;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr bool WIDE = NDS > 3;
+    __shared__ RecG<WIDE> srec[FWD_WARPS][32];
+    const int n = a.T * a.G;
+    const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
+    const int k_beg = split / a.nsub * kchunk, k_end = min(a.K, k_beg + kchunk);
     // this warp's (toy, group) and segment: the last i with segoff[i] <= gw (a warp-uniform search)
     const int gw = blockIdx.x * FWD_WARPS + warp;
-    const int n = a.T * a.G;
     if (gw >= a.segoff[n]) return;
     int lo = 0, hi = n;
     while (hi - lo > 1) {
@@ -352,11 +441,10 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
         if (a.segoff[mid] <= gw) lo = mid; else hi = mid;
     }
     const int t = lo / a.G, g = lo % a.G;
-    constexpr bool WIDE = NDS > 3;
-    __shared__ RecG<WIDE> srec[FWD_WARPS][32];
     int wlo, whi;
     toy_window_union<FAST>(a, t, g, wlo, whi);
     const int j0 = wlo + (gw - a.segoff[lo]) * 64;
+    if (j0 < tb_g_jlin<FAST>(a, g)) return;  // (k_forward_low)
     const int jj[2] = {j0 + lane, j0 + 32 + lane};
     const bool valid[2] = {jj[0] < whi, jj[1] < whi};
     const int nb[2] = {tb_g_node_off<FAST>(a, g) + min(jj[0], whi - 1), tb_g_node_off<FAST>(a, g) + min(jj[1], whi - 1)};
@@ -364,46 +452,13 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
     const float xlo_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + j0];
     const float xhi_w = (float)a.edges[tb_g_edge_off<FAST>(a, g) + jl + 1];
     const int nds = tb_g_nds<FAST>(a, g);
-    const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
-    const int k_beg = split * kchunk, k_end = min(a.K, k_beg + kchunk);
-    const float* blk = reinterpret_cast<const float*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
-
-    // column range of the band: first and last 256-column block that overlaps
-    int kfirst = k_end, klast = k_beg;
-    for (int b = k_beg / COLBLK; b * COLBLK < k_end; ++b) {
-        if (blk[2 * b + 1] < xlo_w || blk[2 * b] > xhi_w) continue;
-        kfirst = min(kfirst, max(b * COLBLK, k_beg));
-        klast = max(klast, min((b + 1) * COLBLK, k_end));
-    }
+    int kfirst, klast;
+    band_columns(a, t, g, k_beg, k_end, xlo_w, xhi_w, kfirst, klast);
+    share_batches(split % a.nsub, a.nsub, kfirst, klast);
 
     double accd[2][MAXGDS] = {};
     int ncol = 0;
-    if (j0 < tb_g_jlin<FAST>(a, g)) {
-        // the warp holds bins below the first linear bin: general node table, one half at a time
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned char cls = a.bclass[nb[h]];
-            const float* nodes = a.ntab_f + (long long)nb[h] * 3 * NGM_F;
-            const float xc = a.xc_f[nb[h]];
-            float del[NG_LOG_F], lam[NG_LOG_F], wt[NG_LOG_F];
-#pragma unroll
-            for (int n = 0; n < NG_LOG_F; ++n) {
-                del[n] = nodes[n]; lam[n] = nodes[NGM_F + n]; wt[n] = valid[h] ? nodes[2 * NGM_F + n] : 0.f;
-            }
-            int nc = 0;
-            for (int k = kfirst; k < klast; ++k) {
-                const float* c = colrec<float>(a, t, g, k);
-                if (c[F_XMAX] < xlo_w || c[F_XMIN] > xhi_w) continue;
-                ++nc;
-                float v = bin_value_f<1, NG_LOG_F>(c, xc, del, lam, wt);
-                if (cls == BIN_ZERO) v = valid[h] ? zerorec<float>(a, t, g, k)[Z_P0] : 0.0f;
-#pragma unroll
-                for (int dd = 0; dd < MAXGDS; ++dd)
-                    if (dd < nds) accd[h][dd] += (double)(v * c[F_TN0 + dd]);
-            }
-            ncol = nc;
-        }
-    } else {
+    {
         const float4 a0 = reinterpret_cast<const float4*>(a.btab_f)[2 * nb[0]];
         const float4 a1 = reinterpret_cast<const float4*>(a.btab_f)[2 * nb[0] + 1];
         const float4 b0 = reinterpret_cast<const float4*>(a.btab_f)[2 * nb[1]];
@@ -476,7 +531,7 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
         const unsigned bins = __popc(__ballot_sync(0xffffffffu, valid[0])) + __popc(__ballot_sync(0xffffffffu, valid[1]));
         if (lane == 0) atomicAdd(&a.work[K_FORWARD], (unsigned long long)ncol * bins);
     }
-    double* out = a.mubuf + ((long long)t * a.nsplit + split) * a.total_bins;
+    double* out = a.mubuf + ((long long)t * a.nrow + split) * a.total_bins;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         if (!valid[h]) continue;
@@ -490,7 +545,7 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
 
 // resident 256-thread blocks per SM the adjoint's register budget is sized for
 #ifndef GSN_BW_MINBLOCKS
-#define GSN_BW_MINBLOCKS 4
+#define GSN_BW_MINBLOCKS 5
 #endif
 
 // SEC: the context has secondary observables (section 2.4): every pair of a bin j that lies in an
@@ -498,9 +553,11 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
 // batches of linear bins then end at the slices' edges, so the added weight is one per-column value
 // per batch.
 // Groups of three or four datasets keep twice as many accumulators: their adjoint gets the register
-// budget of three resident blocks (80 registers; at 64 it spilled ~300 bytes per thread).
+// budget of three resident blocks (80 registers; at 64 it spilled ~300 bytes per thread).  One or two
+// datasets run best with five (48 registers): 4096 toys 34.4 ms with four, 33.7 with five, 38.6 with six;
+// the secondary variant, which needs more, keeps four.
 template <int RES, int NDS, bool FAST, bool SEC>
-__global__ void __launch_bounds__(256, NDS > 2 ? 3 : GSN_BW_MINBLOCKS) k_backward_m(KArgs a) {
+__global__ void __launch_bounds__(256, NDS > 2 ? 3 : SEC ? 4 : GSN_BW_MINBLOCKS) k_backward_m(KArgs a) {
     const int task = blockIdx.x, g = blockIdx.y, t = blockIdx.z;
     if (!tb_g_active<FAST>(a, g)) return;  // no smeared species in the group
     const int W = a.bw_warps;
@@ -1019,14 +1076,18 @@ static cudaError_t launch_fwd(const KArgs& a, cudaStream_t st, int nds) {
         // have (a.ntile * 32 FWD_WARPS >= Jmax bins), and blocks past the last segment return at once
         k_fwd_segments<FAST><<<1, 1024, 0, st>>>(a);
         const long long nseg_max = (long long)a.T * a.G * ((a.ntile * FWD_WARPS * 32 + 63) / 64);
-        dim3 grid((unsigned)((nseg_max + FWD_WARPS - 1) / FWD_WARPS), a.nsplit, 1);
+        dim3 grid((unsigned)((nseg_max + FWD_WARPS - 1) / FWD_WARPS), a.nrow, 1);
+        if (a.jlin_max > 0)
+            k_forward_low<1, 2><<<dim3((a.jlin_max + 63) / 64, a.nsplit, a.T * a.G), FWD_WARPS * 32, 0, st>>>(a);
         if (nds == 1) k_forward_m2<1, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else if (nds == 2) k_forward_m2<2, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else if (nds == 3) k_forward_m2<3, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else k_forward_m2<4, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         return cudaGetLastError();
     }
-    dim3 grid(a.ntile, a.nsplit, a.T * a.G);
+    dim3 grid(a.ntile, a.nrow, a.T * a.G);
+    if (a.jlin_max > 0)
+        k_forward_low<RES, 1><<<dim3((a.jlin_max + 31) / 32, a.nsplit, a.T * a.G), FWD_WARPS * 32, 0, st>>>(a);
     if (nds == 1) k_forward_m<RES, 1, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
     else if (nds == 2) k_forward_m<RES, 2, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
     else if (nds == 3) k_forward_m<RES, 3, FAST><<<grid, FWD_WARPS * 32, 0, st>>>(a);
