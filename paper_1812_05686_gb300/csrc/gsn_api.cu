@@ -451,7 +451,7 @@ int finalize(gsn_ctx* c) {
             if (c->kind[s] < GSN_ANA_PEAK && rfac[(size_t)d * c->S + s] != 0.0) tb.ds_resp[d] = 1;
         }
     // Monte Carlo templates, datasets in order: species, offset, normalised histogram
-    std::vector<int> tpl_s;
+    std::vector<int> tpl_s, tpl_d;
     std::vector<long long> tpl_off;
     std::vector<double> tpl_h;
     for (int d = 0; d < c->D; ++d) {
@@ -460,6 +460,7 @@ int finalize(gsn_ctx* c) {
             const auto it = c->tpl.find(std::make_pair(d, s));
             if (it == c->tpl.end() || rfac[(size_t)d * c->S + s] == 0.0) continue;
             tpl_s.push_back(s);
+            tpl_d.push_back(d);
             tpl_off.push_back((long long)tpl_h.size());
             tpl_h.insert(tpl_h.end(), it->second.begin(), it->second.end());
         }
@@ -626,8 +627,16 @@ int finalize(gsn_ctx* c) {
     }
     if ((rc = upload(c, rfac, &a.rfac))) return rc;
     if ((rc = upload(c, tpl_s, &a.tpl_s))) return rc;
+    if ((rc = upload(c, tpl_d, &a.tpl_d))) return rc;
     if ((rc = upload(c, tpl_off, &a.tpl_off))) return rc;
     if ((rc = upload(c, tpl_h, &a.tpl))) return rc;
+    if (mixed) {
+        std::vector<float> tp;
+        for (double v : tpl_h) put_pair(tp, v);
+        const float* q;
+        if ((rc = upload(c, tp, &q))) return rc;
+        a.tplp = (const float2*)q;
+    }
     if ((rc = upload(c, edges_all, &a.edges))) return rc;
     if ((rc = upload(c, bcls, &a.bclass))) return rc;
     if (mixed) {

@@ -113,8 +113,10 @@ struct KArgs {
                                 // and adjoint are skipped: a pure template fit)
     int ntpl;                   // Monte Carlo templates over all datasets
     const int* tpl_s;           // [ntpl] species of each template (datasets in order)
+    const int* tpl_d;           // [ntpl] its dataset
     const long long* tpl_off;   // [ntpl] offset of its normalised histogram in tpl
     const double* tpl;          // concatenated histograms, n_bins of the template's dataset each
+    const float2* tplp;         // the same as FP32 pairs (mixed)
     FastTables ft;
     // device-resident problem arrays
     const Tables* tb;

@@ -663,6 +663,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
     const long long sstride = a.total_bins;
     const double* mrow = a.mubuf + (long long)t * a.nrow * a.total_bins;
     double part = 0.0;
+    float ph = 0.f, pl = 0.f;   // the terms that pairs hold
     int bad_mu = 0, bad_fin = 0;
     for (int d = 0; d < a.D; ++d) {
         const int J = tb_ds_bins(a, d), off = tb_ds_off(a, d);
@@ -709,7 +710,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                 }
             }
             if (j >= j1) continue;
-            double w = 0.0;
+            R w = 0;
             if (j >= lo && j < hi) {
                 double mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
                 if constexpr (sizeof(R) == 8) {
@@ -728,20 +729,52 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                 }
                 for (int q = 0; q < ntp; ++q) mu = fma(tcoef[q], a.tpl[toff[q] + j], mu);
                 const double n = cnt[off + j];
-                double term;
-                if (n > 0.0) {
-                    if (!(mu > 0.0)) { bad_mu = 1; term = INFINITY; }
-                    else term = mu - n + n * log(n / mu);
+                float th, tl;
+                if (n > 0.0 && poisson_term(mu, n, th, tl)) {
+                    acc_pair(ph, pl, th, tl);
+                    if constexpr (sizeof(R) == 4) {
+                        // w = (mu - n) / mu, the FP32 value the adjoint reads
+                        const float2 e = split(n - mu), m = split(mu);
+                        float q, qe;
+                        div_pair(-e.x, -e.y, m.x, m.y, q, qe);
+                        w = q + qe;
+                    } else {
+                        w = 1.0 - n / mu;
+                    }
                 } else {
-                    term = mu;
+                    double term = mu;
+                    if (n > 0.0) {
+                        if (!(mu > 0.0)) { bad_mu = 1; term = INFINITY; }
+                        else term = mu - n + n * log(n / mu);
+                    }
+                    if (!isfinite(mu)) bad_fin = 1;
+                    part += term;
+                    w = mu > 0.0 ? (R)(1.0 - n / mu) : R(0);
                 }
-                if (!isfinite(mu)) bad_fin = 1;
-                part += term;
-                w = mu > 0.0 ? 1.0 - n / mu : 0.0;
             }
-            wout[off + j] = (R)w;
+            wout[off + j] = w;
         }
-        // template rate gradients: this block's share of sum_j w_j T_j (w as the adjoint reads it)
+        // template rate gradients: this block's share of sum_j w_j T_j (w as the adjoint reads it).  Mixed:
+        // w is FP32, the products and sums are pairs (48 bits), a warp per template
+        if (sizeof(R) == 4 && ntp > 0) {
+            __syncthreads();  // w of every thread
+            const int ja = max(j0, lo), jb = min(j1, hi);
+            for (int q = threadIdx.x >> 5; q < ntp; q += blockDim.x >> 5) {
+                const float2* T = a.tplp + toff[q];
+                const R* wd = wout + off;
+                float gh = 0.f, gl = 0.f;
+#pragma unroll 4
+                for (int j = ja + (threadIdx.x & 31); j < jb; j += 32) {
+                    const float2 T2 = T[j];
+                    float p, e;
+                    mul_pair((float)wd[j], 0.f, T2.x, T2.y, p, e);
+                    acc_pair(gh, gl, p, e);
+                }
+                const double g = warp_sum<double>(join(gh, gl));
+                if ((threadIdx.x & 31) == 0) dp[2 + a.tb->ds_tpl0[d] + q] = g;
+            }
+            continue;
+        }
         for (int q = 0; q < ntp; ++q) {
             double gpart = 0.0;
             for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
@@ -752,7 +785,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
             if (threadIdx.x == 0) dp[2 + a.tb->ds_tpl0[d] + q] = gpart;
         }
     }
-    const double sum = block_sum_d(part, sh);
+    const double sum = block_sum_d(part + join(ph, pl), sh);
     const int any_bad_mu = __syncthreads_or(bad_mu), any_bad_fin = __syncthreads_or(bad_fin);
     if (threadIdx.x == 0) {
         dp[0] = sum;
@@ -806,24 +839,38 @@ __global__ void __launch_bounds__(256) k_devfinal(KArgs a) {
             }
         }
     }
+    const int pstride = 2 + a.ntpl;
+    const double* dp = a.devpart + (long long)t * a.dev_chunks * pstride;
+    if (a.want_grad && a.ntpl > 0) {
+        // Monte Carlo template rates: d mu_dj / d r_s = eps_d f_ds T_dsj; a thread per template, then
+        // every parameter adds its own in order (one thread walking them took 30 us per block)
+        __shared__ double sg[256];
+        __shared__ int sp[256];
+        for (int q0 = 0; q0 < a.ntpl; q0 += 256) {
+            const int gq = q0 + threadIdx.x;
+            __syncthreads();
+            sp[threadIdx.x] = -1;
+            if (gq < a.ntpl) {
+                const int d = a.tpl_d[gq], s = a.tpl_s[gq];
+                double g = 0.0;
+                for (int c = 0; c < a.dev_chunks; ++c) g += dp[pstride * c + 2 + gq];
+                sg[threadIdx.x] = a.rfac[d * a.S + s] * g;
+                sp[threadIdx.x] = a.slot_map[d * a.NSLOT + s];
+            }
+            __syncthreads();
+            for (int p = threadIdx.x; p < a.P; p += 256) {
+                double g = gdir[p];
+                for (int i = 0; i < min(256, a.ntpl - q0); ++i)
+                    if (sp[i] == p) g += sg[i];
+                gdir[p] = g;
+            }
+        }
+        __syncthreads();  // gdir before thread 0 adds the pulls
+    }
     if (threadIdx.x == 0) {
-        const int pstride = 2 + a.ntpl;
-        const double* dp = a.devpart + (long long)t * a.dev_chunks * pstride;
         double nll = 0.0;
         int flags = 0;
         for (int c = 0; c < a.dev_chunks; ++c) { nll += dp[pstride * c]; flags |= (int)dp[pstride * c + 1]; }
-        if (a.want_grad && a.ntpl > 0) {
-            // Monte Carlo template rates: d mu_dj / d r_s = eps_d f_ds T_dsj
-            for (int d = 0; d < a.D; ++d)
-                for (int q = 0; q < a.tb->ds_ntpl[d]; ++q) {
-                    const int gq = a.tb->ds_tpl0[d] + q, s = a.tpl_s[gq];
-                    const int p = a.slot_map[d * a.NSLOT + s];
-                    if (p < 0) continue;
-                    double g = 0.0;
-                    for (int c = 0; c < a.dev_chunks; ++c) g += dp[pstride * c + 2 + gq];
-                    gdir[p] += a.rfac[d * a.S + s] * g;
-                }
-        }
         // secondary-observable pieces (section 2.4): NLL, flags and slot gradients per dataset
         for (int i = 0; i < a.nsec; ++i) {
             const double* sp = a.secpart + ((long long)t * a.nsec + i) * (2 + a.NSLOT);

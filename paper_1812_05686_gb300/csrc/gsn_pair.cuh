@@ -1,6 +1,6 @@
 // Records of the FP64 response kernels that work in pairs of FP32 numbers (gsn_pair64.cu).
 #pragma once
-#include "gsn_internal.cuh"
+#include "gsn_device.cuh"
 
 namespace gsn {
 
@@ -33,5 +33,73 @@ struct __align__(16) PairRec {
     float2 T[MAXGDS];
 };
 static_assert(sizeof(PairRec) == 96, "three sectors");
+
+// ------------------------------------------------ arithmetic on pairs -----
+// TwoSum of a running pair (sh, sl) and p, error terms collected in sl
+DEV void acc_pair(float& sh, float& sl, float p, float e) {
+    const float t = __fadd_rn(sh, p);
+    const float bp = __fsub_rn(t, sh);
+    const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
+    sl = __fadd_rn(sl, __fadd_rn(er, e));
+    sh = t;
+}
+// (s, l) with l brought below half an ulp of s
+DEV void renorm(float& s, float& l) {
+    const float t = __fadd_rn(s, l);
+    l = __fsub_rn(l, __fsub_rn(t, s));
+    s = t;
+}
+// product of two pairs: leading part p, the rest e
+DEV void mul_pair(float ah, float al, float bh, float bl, float& p, float& e) {
+    p = __fmul_rn(ah, bh);
+    e = fmaf(ah, bh, -p);
+    e = fmaf(ah, bl, fmaf(al, bh, e));
+}
+DEV float2 split(double v) {
+    const float h = (float)v;
+    return make_float2(h, (float)(v - (double)h));
+}
+DEV double join(float h, float l) { return (double)h + (double)l; }
+// a / b to ~2^-46
+DEV void div_pair(float ah, float al, float bh, float bl, float& q, float& e) {
+    const float r = __frcp_rn(bh);
+    q = __fmul_rn(ah, r);
+    e = __fmul_rn(fmaf(-q, bl, __fadd_rn(fmaf(-q, bh, ah), al)), r);
+}
+
+// Poisson term mu - n + n ln(n / mu) of Eq. (LL) for counts and expectation that differ by less than a
+// factor 1.5, without the FP64 logarithm and division (~100 FP64-pipe operations of 64 cycles): with
+// e = n - mu and u = e / (n + mu),
+//     term = u (e + (n + mu + e) v S),  v = u^2,  S = 1/3 + v/5 + v^2/7 + ...
+// in which nothing cancels (mu - n + n ln(n / mu) loses n 2^-53 to the rounding of n / mu).  Pairs hold
+// S's first five terms; the rest, v^5 (1/13 + ...) < 8e-9, is FP32.  False outside the range.
+DEV bool poisson_term(double mu, double n, float& th, float& tl) {
+    const double e = n - mu, s = n + mu;
+    const float2 E = split(e), A = split(s);
+    if (!(fabsf(E.x) <= 0.2f * A.x) || !(A.x > 1e-30f && A.x < 1e30f)) return false;
+    float uh, ul, vh, vl, p, q, yh, yl;
+    div_pair(E.x, E.y, A.x, A.y, uh, ul);
+    mul_pair(uh, ul, uh, ul, vh, vl);
+    float R = fmaf(vh, 1.0f / 19, 1.0f / 17);
+    R = fmaf(R, vh, 1.0f / 15);
+    R = fmaf(R, vh, 1.0f / 13);
+    constexpr double c[5] = {1.0 / 3, 1.0 / 5, 1.0 / 7, 1.0 / 9, 1.0 / 11};
+    yh = R; yl = 0.f;
+#pragma unroll
+    for (int i = 4; i >= 0; --i) {   // y <- c_i + v y
+        mul_pair(yh, yl, vh, vl, p, q);
+        const float ch = (float)c[i], cl = (float)(c[i] - (double)ch);
+        yh = ch; yl = cl;
+        acc_pair(yh, yl, p, q);
+    }
+    mul_pair(yh, yl, vh, vl, p, q);
+    float mh = A.x, ml = A.y;        // 2 n
+    acc_pair(mh, ml, E.x, E.y);
+    mul_pair(mh, ml, p, q, yh, yl);
+    mh = E.x; ml = E.y;
+    acc_pair(mh, ml, yh, yl);
+    mul_pair(mh, ml, uh, ul, th, tl);
+    return true;
+}
 
 }  // namespace gsn

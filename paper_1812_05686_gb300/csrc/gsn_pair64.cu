@@ -49,32 +49,6 @@ namespace {
 
 constexpr int PW = 8;   // warps per block of the forward
 
-// TwoSum of a running pair (sh, sl) and p, error terms collected in sl
-DEV void acc_pair(float& sh, float& sl, float p, float e) {
-    const float t = __fadd_rn(sh, p);
-    const float bp = __fsub_rn(t, sh);
-    const float er = __fadd_rn(__fsub_rn(sh, __fsub_rn(t, bp)), __fsub_rn(p, bp));
-    sl = __fadd_rn(sl, __fadd_rn(er, e));
-    sh = t;
-}
-// (s, l) with l brought below half an ulp of s
-DEV void renorm(float& s, float& l) {
-    const float t = __fadd_rn(s, l);
-    l = __fsub_rn(l, __fsub_rn(t, s));
-    s = t;
-}
-// product of two pairs: leading part p, the rest e
-DEV void mul_pair(float ah, float al, float bh, float bl, float& p, float& e) {
-    p = __fmul_rn(ah, bh);
-    e = fmaf(ah, bh, -p);
-    e = fmaf(ah, bl, fmaf(al, bh, e));
-}
-DEV float2 split(double v) {
-    const float h = (float)v;
-    return make_float2(h, (float)(v - (double)h));
-}
-DEV double join(float h, float l) { return (double)h + (double)l; }
-
 // 2^(s + lo), times the power of two whose exponent bits nb holds, as an FP32 pair; |s| < 4096
 DEV void pair_exp2(float s, float lo, int nb, const float2* __restrict__ tab, float& vh, float& vl) {
     // s = n/1024 + r: the table holds 2^(i/1024), and |r| < 2^-11 leaves a cubic
