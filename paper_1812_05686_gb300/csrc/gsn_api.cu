@@ -67,6 +67,9 @@ struct gsn_ctx {
     // scratch
     Buf secRq_b, secN_b, secV_b, secW_b, secpart_b, secU_b;  // per-toy buffers of the secondary pieces
     Buf segbuf;              // forward segment prefix [T*G + 1]
+    Buf point_b;             // single-point results: NLL, status, gradient
+    double* host = nullptr;  // pinned staging of the single-point calls
+    size_t host_n = 0;
     Buf sppart;              // FP64 in pairs: per-species partial sums
     Buf pairbuf, batbuf, fbuf, wfbuf, hvybuf;  // FP64 in pairs: column records, batch summaries, centre sums,
                              // filtered weights, heavy columns
@@ -124,6 +127,21 @@ int ensure(gsn_ctx* c, Buf& b, size_t bytes) {
         return fail(c, GSN_ERR_NOMEM, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
     }
     b.n = bytes;
+    ++c->scratch_gen;
+    return GSN_OK;
+}
+
+// pinned host staging of the single-point calls (n doubles)
+int ensure_host(gsn_ctx* c, size_t n) {
+    if (c->host && c->host_n >= n) return GSN_OK;
+    if (c->host) cudaFreeHost(c->host);
+    c->host = nullptr; c->host_n = 0;
+    if (cudaMallocHost((void**)&c->host, n * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        c->host = nullptr;
+        return fail(c, GSN_ERR_NOMEM, "cudaMallocHost of " + std::to_string(n * sizeof(double)) + " bytes failed");
+    }
+    c->host_n = n;
     ++c->scratch_gen;
     return GSN_OK;
 }
@@ -1154,13 +1172,14 @@ void gsn_destroy(gsn_ctx* c) {
     for (Buf* b : {&c->fit_ws, &c->fit_cfg, &c->fit_eval, &c->fit_ist, &c->wscale_b, &c->rfit_cfg, &c->rfit_ws})
         if (b->p) cudaFree(b->p);
     for (Buf* b : {&c->secRq_b, &c->secN_b, &c->secV_b, &c->secW_b, &c->secpart_b, &c->secU_b,
-                   &c->sppart, &c->hvybuf, &c->pairbuf, &c->batbuf, &c->fbuf, &c->wfbuf, &c->segbuf, &c->zerobuf, &c->colbuf, &c->colbuf2, &c->blkbuf, &c->mubuf, &c->wbuf, &c->partbuf, &c->gdirect, &c->devbuf, &c->params, &c->counts_b,
+                   &c->point_b, &c->sppart, &c->hvybuf, &c->pairbuf, &c->batbuf, &c->fbuf, &c->wfbuf, &c->segbuf, &c->zerobuf, &c->colbuf, &c->colbuf2, &c->blkbuf, &c->mubuf, &c->wbuf, &c->partbuf, &c->gdirect, &c->devbuf, &c->params, &c->counts_b,
                    &c->win_b, &c->nll_b, &c->grad_b, &c->status_b, &c->Mbuf, &c->outbuf, &c->s_hi, &c->s_lo,
                    &c->tc_part, &c->tc_err})
         if (b->p) cudaFree(b->p);
     if (c->work.p) cudaFree(c->work.p);
     for (auto& p : c->pending) { c->event_pool.push_back(p.e0); c->event_pool.push_back(p.e1); }
     for (cudaEvent_t e : c->event_pool) cudaEventDestroy(e);
+    if (c->host) cudaFreeHost(c->host);
     if (c->aux) { cudaStreamSynchronize(c->aux); cudaStreamDestroy(c->aux); }
     if (c->fork_ev) cudaEventDestroy(c->fork_ev);
     if (c->join_ev) cudaEventDestroy(c->join_ev);
@@ -1456,26 +1475,41 @@ int gsn_eval_grad(gsn_ctx* c, const double* params, double* nll, double* grad) {
     if ((rc = finalize(c))) return rc;
     if (!nll) return fail(c, GSN_ERR_ARG, "nll is NULL");
     if ((rc = check_params_host(c, params))) return rc;
-    if ((rc = ensure(c, c->params, c->P * sizeof(double)))) return rc;
-    if ((rc = ensure(c, c->nll_b, sizeof(double)))) return rc;
-    if ((rc = ensure(c, c->grad_b, c->P * sizeof(double)))) return rc;
-    if ((rc = ensure(c, c->status_b, sizeof(int)))) return rc;
-    CUDA_TRY(c, cudaMemcpyAsync(c->params.p, params, c->P * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    // one pinned buffer and one device buffer, so that the copies are part of the captured sequence:
+    // parameters in, (NLL, status, gradient) out.  Four pageable copies per call, each staged by the
+    // driver, cost more than the kernels of a small fit
+    const size_t P = c->P, nout = 2 + (grad ? P : 0);
+    if ((rc = ensure(c, c->params, P * sizeof(double)))) return rc;
+    if ((rc = ensure(c, c->point_b, (P + 2) * sizeof(double)))) return rc;
+    if ((rc = ensure_host(c, 2 * P + 2))) return rc;
+    double *hin = c->host, *hout = c->host + P, *out = (double*)c->point_b.p;
+    std::memcpy(hin, params, P * sizeof(double));
     KArgs a = c->base;
     a.params = (const double*)c->params.p; a.params_stride = c->P;
     a.counts_stride = 0; a.win_stride = 0;
-    a.nll = (double*)c->nll_b.p; a.grad = grad ? (double*)c->grad_b.p : nullptr; a.status = (int*)c->status_b.p;
+    a.nll = out; a.status = (int*)(out + 1); a.grad = grad ? out + 2 : nullptr;
     a.want_grad = grad ? 1 : 0;
+    auto copy_in = [&]() -> int {
+        CUDA_TRY(c, cudaMemcpyAsync(c->params.p, hin, P * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+        return GSN_OK;
+    };
+    if (c->tuned.find({1, grad ? 1 : 0}) == c->tuned.end() && (rc = copy_in())) return rc;  // the tuner's inputs
     Plan p;
     if ((rc = choose_plan(c, 1, a, grad != nullptr, p))) return rc;
     if ((rc = prepare(c, 1, p, a))) return rc;
     const std::vector<long long> key = {2, grad ? 1 : 0, p.nsplit, p.bw_warps, p.bw_bsplit, p.dev_chunks};
-    if ((rc = replay(c, key, [&]() { return run_step(c, a, grad != nullptr); }))) return rc;
-    int st = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(nll, c->nll_b.p, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    if (grad) CUDA_TRY(c, cudaMemcpyAsync(grad, c->grad_b.p, c->P * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(&st, c->status_b.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    rc = replay(c, key, [&]() -> int {
+        int r;
+        if ((r = copy_in()) || (r = run_step(c, a, grad != nullptr))) return r;
+        CUDA_TRY(c, cudaMemcpyAsync(hout, out, nout * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        return GSN_OK;
+    });
+    if (rc) return rc;
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    *nll = hout[0];
+    int st;
+    std::memcpy(&st, hout + 1, sizeof st);
+    if (grad) std::memcpy(grad, hout + 2, P * sizeof(double));
     return status_message(c, st, 0);
 }
 
@@ -1580,9 +1614,10 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     if (!nll) return fail(c, GSN_ERR_ARG, "nll is NULL");
     if ((rc = check_params_host(c, params))) return rc;
     if ((rc = ensure(c, c->params, c->P * sizeof(double)))) return rc;
-    if ((rc = ensure(c, c->nll_b, sizeof(double)))) return rc;
-    if ((rc = ensure(c, c->status_b, sizeof(int)))) return rc;
-    CUDA_TRY(c, cudaMemcpyAsync(c->params.p, params, c->P * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+    if ((rc = ensure(c, c->point_b, (c->P + 2) * sizeof(double)))) return rc;
+    if ((rc = ensure_host(c, 2 * (size_t)c->P + 2))) return rc;
+    std::memcpy(c->host, params, c->P * sizeof(double));
+    CUDA_TRY(c, cudaMemcpyAsync(c->params.p, c->host, c->P * sizeof(double), cudaMemcpyHostToDevice, c->stream));
     bool hit = false;
     if ((rc = species_cached(c, params, hit))) return rc;
     KArgs a = c->base;
@@ -1592,7 +1627,7 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     a.params = (const double*)c->params.p; a.params_stride = c->P;
     a.counts_stride = 0; a.win_stride = 0;
     a.Mbuf = (double*)c->Mbuf.p;
-    a.nll = (double*)c->nll_b.p; a.grad = nullptr; a.status = (int*)c->status_b.p;
+    a.nll = (double*)c->point_b.p; a.grad = nullptr; a.status = (int*)(a.nll + 1);
     a.want_grad = 0;
     a.Mbuf = (double*)c->Mbuf.p;  // the cached shapes (one parameter point)
     a.secRq = nullptr;            // the secondary pieces take their slice sums from them
@@ -1601,10 +1636,12 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     if (a.nsec && (rc = launch(c, K_SPECIES, a, launch_secondary))) return rc;
     if ((rc = launch(c, K_DEVIANCE, a, launch_deviance))) return rc;
     if ((rc = launch(c, K_DEVFINAL, a, launch_devfinal))) return rc;
-    int st = 0;
-    CUDA_TRY(c, cudaMemcpyAsync(nll, c->nll_b.p, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_TRY(c, cudaMemcpyAsync(&st, c->status_b.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    double* hout = c->host + c->P;
+    CUDA_TRY(c, cudaMemcpyAsync(hout, c->point_b.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+    *nll = hout[0];
+    int st;
+    std::memcpy(&st, hout + 1, sizeof st);
     if (!hit && (rc = species_status(c))) return rc;
     return status_message(c, st, 0);
 }

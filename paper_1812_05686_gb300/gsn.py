@@ -411,8 +411,11 @@ def make_autograd():
             rc, nll, g = ctx.eval_grad(params.detach().cpu().double().numpy())
             if rc != GSN_OK:
                 raise GsnError(rc, ctx.last_error())
-            fctx.save_for_backward(torch.from_numpy(g).to(params.device, params.dtype))
-            return torch.tensor(nll, dtype=params.dtype, device=params.device)
+            # one transfer for the NLL and the gradient; the NLL gets storage of its own, so that an
+            # in-place operation on the loss leaves the saved gradient alone
+            out = torch.from_numpy(np.append(g, nll)).to(params.device, params.dtype)
+            fctx.save_for_backward(out[:-1])
+            return out[-1].clone()
 
         @staticmethod
         def backward(fctx, gout):
