@@ -64,6 +64,20 @@ DEV void gg_H_Hx(double x, double a, double& H, double& Hx) {
     Hx = hx;
 }
 
+// Constants of a toy's power p that every column shares, made once per block (as per-column divisions and
+// logarithms they were a tenth of the prologue's FP64 operations; the same operations, so the same bits)
+struct GGPower { double p, a, b2, b3, b4, lnp; };
+DEV GGPower gg_power(double p) {
+    GGPower c;
+    c.p = p;
+    c.a = 1.0 / p;
+    c.b2 = 0.5 - c.a;
+    c.b3 = (1.0 + c.a * (7.0 * c.a - 6.0)) / 6.0;
+    c.b4 = -c.a * (2.0 + c.a * (6.0 * c.a - 7.0)) / 4.0;
+    c.lnp = log(p);
+    return c;
+}
+
 // x = d/p solving H(x) = r = ln(1 + var/mu^2): Newton's method on ln H against ln x, started from
 // the series reversion of the first four terms of H's large-x expansion (Stirling's series with the
 // Bernoulli polynomials B_2..B_5; a = 1 gives ln(1 + 1/x)),
@@ -72,8 +86,8 @@ DEV void gg_H_Hx(double x, double a, double& H, double& Hx) {
 // below 1e-7 (the error left is its square).  lnx = ln x; hx = dH/dx at the root (the value at the
 // last point evaluated, moved to the root with dHx/dx = -2 Hx / x of the leading term).  Returns a
 // negative value if it fails.
-DEV double gg_solve_shape(double r, double a, double& lnx, double& hx) {
-    const double b2 = 0.5 - a, b3 = (1.0 + a * (7.0 * a - 6.0)) / 6.0, b4 = -a * (2.0 + a * (6.0 * a - 7.0)) / 4.0;
+DEV double gg_solve_shape(double r, const GGPower& pc, double& lnx, double& hx) {
+    const double a = pc.a, b2 = pc.b2, b3 = pc.b3, b4 = pc.b4;
     const double y0 = r / (a * a);
     const double y = y0 * (1.0 + y0 * (-b2 + y0 * ((2.0 * b2 * b2 - b3) + y0 * (b2 * (5.0 * b3 - 5.0 * b2 * b2) - b4))));
     double x = 1.0 / y;
@@ -184,12 +198,12 @@ DEV void gg_inc_gamma(double a, double y, double& P, double& Pa, double& py) {
 // lfmu, kappa1, Amu: ln f(mu), kappa_1 and (mu/s)^p.  Returns the normalisation N_k that multiplies the T_dk (mixed: the density at the mean times
 // ex2_scale = 1 / (1 + b), b the SFU exponentials' measured mean relative error; FP64: 1).
 template <class R>
-DEV double gg_column(double mu, double var, double p, double cut, double x1, bool zero_bin, bool mixed,
+DEV double gg_column(double mu, double var, const GGPower& pc, double cut, double x1, bool zero_bin, bool mixed,
                      double ex2_scale, R* f, R* z, double* gco, R& xmin, R& xmax, double& lfmu, double& kappa1, double& Amu) {
-    const double a = 1.0 / p;
+    const double p = pc.p, a = pc.a;
     const double r = log1p(var / (mu * mu));
     double Hx, lxs;                                   // dH/dx at the root, ln(d/p)
-    const double xs = gg_solve_shape(r, a, lxs, Hx);  // d/p
+    const double xs = gg_solve_shape(r, pc, lxs, Hx);  // d/p
     const double d = p * xs;
     double ls, psi, lgx, da;                          // ln(mu/s), psi(d/p), lnGamma(d/p), psi(d/p + a) - psi(d/p)
     gg_at_shape(xs, lxs, a, ls, psi, lgx, da);
@@ -197,7 +211,7 @@ DEV double gg_column(double mu, double var, double p, double cut, double x1, boo
     const double A = exp(p * ls);                     // (mu/s)^p
     const double k1 = (d - 1.0) - p * A;
     // density at the mean: ln f(mu) = ln p - ln mu + d ln(mu/s) - A - lnGamma(d/p)
-    const double lfm = log(p) - log(mu) + d * ls - A - lgx;
+    const double lfm = pc.lnp - log(mu) + d * ls - A - lgx;
     lfmu = lfm; kappa1 = k1; Amu = A;
     double Nk = 1.0;
     if (mixed) {
@@ -206,7 +220,7 @@ DEV double gg_column(double mu, double var, double p, double cut, double x1, boo
         f[F_B] = (R)(1.4426950408889634 * A);
         f[F_C] = (R)(1.4426950408889634 * k1);
     } else {
-        f[F_A] = (R)(log(p) - d * lns - lgx);
+        f[F_A] = (R)(pc.lnp - d * lns - lgx);
         f[F_B] = (R)(d - 1.0);
         f[F_C] = (R)lns;
     }
@@ -257,7 +271,9 @@ DEV double gg_column(double mu, double var, double p, double cut, double x1, boo
         gg_inc_gamma(xs, y, P, Pa, py);
         P0 = P; P0d = Pa / p; P0s = -p * py; P0p = -(d / (p * p)) * Pa + py * lxs;
     }
-    z[Z_P0] = (R)(P0 / Nk);
+    // the bin at zero: most columns do not reach it, and 0 / Nk is 0
+    if (P0 != 0.0) z[Z_P0] = (R)(P0 / Nk);
+    const double P0dN = P0d != 0.0 ? P0d / Nk : 0.0, P0sN = P0s != 0.0 ? P0s / Nk : 0.0, P0pN = P0p != 0.0 ? P0p / Nk : 0.0;
     // moment matching H(x, a) = ln rho, ln s = ln mu - G(x, a): implicit derivatives of x and u = ln s
     // dH/da = 2 [psi(x + 2a) - psi(x + a)] = 2 (dH/dx + [psi(x + a) - psi(x)]): no cancellation
     const double Ha = 2.0 * (Hx + da);
@@ -277,9 +293,9 @@ DEV double gg_column(double mu, double var, double p, double cut, double x1, boo
         m0 = -psi / p; m1 = p; m2 = -d;
         m3 = 1.0 / p + d * psi / (p * p); m4 = -1.0; m5 = 0.0; m6 = 0.0;
     }
-    const double gd[5] = {m0, 1.0, 0.0, 0.0, P0d / Nk};
-    const double gs[5] = {m2, 0.0, m1, 0.0, P0s / Nk};
-    const double gp[5] = {m3 + m6 * m2, m5, m6 * m1, m4, P0p / Nk};
+    const double gd[5] = {m0, 1.0, 0.0, 0.0, P0dN};
+    const double gs[5] = {m2, 0.0, m1, 0.0, P0sN};
+    const double gp[5] = {m3 + m6 * m2, m5, m6 * m1, m4, P0pN};
     double row[3][5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {

@@ -288,6 +288,8 @@ cudaError_t launch_deviance(const KArgs& a, cudaStream_t st);
 cudaError_t launch_devfinal(const KArgs& a, cudaStream_t st);
 cudaError_t launch_backward(const KArgs& a, cudaStream_t st);
 cudaError_t launch_gradfinal(const KArgs& a, cudaStream_t st);
+cudaError_t launch_forward_gg(const KArgs& a, cudaStream_t st);
+cudaError_t launch_backward_gg(const KArgs& a, cudaStream_t st);
 cudaError_t launch_forward_pair(const KArgs& a, cudaStream_t st);
 cudaError_t launch_backward_pair(const KArgs& a, cudaStream_t st);
 cudaError_t launch_species_pair(const KArgs& a, cudaStream_t st);

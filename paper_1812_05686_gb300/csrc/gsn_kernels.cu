@@ -94,6 +94,13 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
     __syncthreads();
     const double LY = sres[0], kB = sres[1], ra = sres[2], rb = sres[3], rc = sres[4];
     const double alpha = 1.0 + kB * a.s0, beta = kB * a.s1;
+    // generalized gamma: constants of the toy's quenching and power, once per block
+    __shared__ GGPower spow;
+    __shared__ double sq[3];   // beta/alpha^2, s0 beta/alpha, alpha^2
+    if (RES == 2 && threadIdx.x == 0) {
+        spow = gg_power(sres[5]);
+        sq[0] = beta / (alpha * alpha); sq[1] = a.s0 * (beta / alpha); sq[2] = alpha * alpha;
+    }
     if (sizeof(R) == 4 && threadIdx.x == 0) {
         const double ia = 1.0 / alpha;
         sdf[0] = (float)ia; sdf[1] = (float)(ia - (double)(float)ia);
@@ -126,18 +133,18 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
             if (beta > 0) {
                 y = alpha * E / beta;
                 L = log1p(y);
-                Eq = y < 1.0 ? -(beta / (alpha * alpha)) * (L - y) : E / alpha - (beta / (alpha * alpha)) * L;
+                Eq = y < 1.0 ? -sq[0] * (L - y) : E / alpha - sq[0] * L;
             }
             const double mud = LY * Eq;
             const double vard = fma(mud, fma(rc, mud, rb), ra);
             psig = sqrt(vard);
             const double D = L - y, r1 = y / (1.0 + y);
-            f[F_DEQ] = (R)(beta > 0 ? (a.s0 * (beta / alpha) * (2.0 * D + y * r1) - a.s1 * (D + y * r1)) / (alpha * alpha) : NAN);
+            f[F_DEQ] = (R)(beta > 0 ? (sq[1] * (2.0 * D + y * r1) - a.s1 * (D + y * r1)) / sq[2] : NAN);
             f[F_MUH] = (R)mud;
             if constexpr (sizeof(R) == 4) f[F_MUL] = (R)(mud - (double)(R)mud);
             double gco[NFG];
             const double x1 = a.edges[tb_g_edge_off<FAST>(a, g) + 1];
-            Nk = (R)gg_column<R>(mud, vard, sres[5], a.cut, x1, tb_g_zero<FAST>(a, g) != 0, sizeof(R) == 4, a.ex2_scale, f, z, gco,
+            Nk = (R)gg_column<R>(mud, vard, spow, a.cut, x1, tb_g_zero<FAST>(a, g) != 0, sizeof(R) == 4, a.ex2_scale, f, z, gco,
                                  xmin, xmax, pfm, pk1, pAp);
             if constexpr (sizeof(R) == 8) plm = log(mud);
             double* g2 = a.colbuf2 + (((long long)t * a.G + g) * a.K + k) * NFG;
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
 // ------------------------------------------------------------- forward -----
 template <class R, int RES, int NG>
 DEV int forward_loop(const KArgs& a, int t, int g, int split, float xlo_w, float xhi_w, bool valid,
-                     bool is_zero, const R* nodes, R xc, double* accd) {
+                     bool is_zero, const R* nodes, R xc, double* accd, int bfirst = 0, int bstep = 1) {
     int ncol = 0;
     const int nds = tb_g_nds(a, g);
     const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
@@ -433,7 +440,7 @@ DEV int forward_loop(const KArgs& a, int t, int g, int split, float xlo_w, float
             del[n] = nodes[n]; lam[n] = nodes[NGM_D + n]; wt[n] = valid ? nodes[2 * NGM_D + n] : R(0);
         }
     }
-    for (int b = k_beg / COLBLK; b * COLBLK < k_end; ++b) {
+    for (int b = k_beg / COLBLK + bfirst; b * COLBLK < k_end; b += bstep) {
         if (blk[2 * b + 1] < (R)xlo_w || blk[2 * b] > (R)xhi_w) continue;
         // FP32: partial sums of up to 32 columns folded into compensated (s, cs) pairs
         R acc[MAXGDS] = {}, sacc[MAXGDS] = {}, cacc[MAXGDS] = {};
@@ -521,6 +528,41 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, (sizeof(R) == 4 && RES == 2) ?
     if (valid) {
         double* out = a.mubuf + ((long long)t * a.nsplit + split) * a.total_bins;
         for (int dd = 0; dd < tb_g_nds(a, g); ++dd) out[tb_ds_off(a, tb_g_ds(a, g, dd)) + j] = accd[dd];
+    }
+}
+
+// Mixed generalized gamma, tiles of 32 bins that hold bins of the general node table (the first of the
+// histogram; the others: k_forward_gg): a block per tile, its warps every eighth block of 256 columns
+// (one warp per tile made the few such tiles of a toy batch the launch's tail: 16.8 -> 14.5 ms per 1024 toys)
+__global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_gg_low(KArgs a) {
+    __shared__ double sred[FWD_WARPS][32];
+    const int split = blockIdx.y, t = blockIdx.z / a.G, g = blockIdx.z % a.G;
+    if (!tb_g_active(a, g)) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int wlo, whi;
+    toy_window_union(a, t, g, wlo, whi);
+    const int j0 = blockIdx.x * 32;
+    if (j0 >= whi || j0 + 32 <= wlo) return;
+    const int j = j0 + lane;
+    const bool valid = j >= wlo && j < whi;
+    const int nb = tb_g_node_off(a, g) + min(max(j, wlo), whi - 1);
+    const unsigned char cls = a.bclass[nb];
+    if (!__any_sync(0xffffffffu, cls != BIN_LIN)) return;
+    const float xlo_w = (float)a.edges[tb_g_edge_off(a, g) + max(j0, wlo)];
+    const float xhi_w = (float)a.edges[tb_g_edge_off(a, g) + min(j0 + 31, whi - 1) + 1];
+    double accd[MAXGDS] = {};
+    const int ncol = forward_loop<float, 2, NG_LOG_F>(a, t, g, split, xlo_w, xhi_w, valid, cls == BIN_ZERO,
+                                                      a.ntab_f + (long long)nb * 3 * NGM_F, a.xc_f[nb], accd, warp, FWD_WARPS);
+    count_work(a, K_FORWARD, valid, ncol);
+    for (int dd = 0; dd < tb_g_nds(a, g); ++dd) {
+        __syncthreads();
+        sred[warp][lane] = accd[dd];
+        __syncthreads();
+        if (warp == 0 && valid) {
+            double v = 0.0;
+            for (int w = 0; w < FWD_WARPS; ++w) v += sred[w][lane];
+            a.mubuf[((long long)t * a.nsplit + split) * a.total_bins + tb_ds_off(a, tb_g_ds(a, g, dd)) + j] = v;
+        }
     }
 }
 
@@ -1631,9 +1673,13 @@ cudaError_t launch_forward(const KArgs& a, cudaStream_t st) {
     if (a.pair) return launch_forward_pair(a, st);
     dim3 grid(a.ntile, a.nsplit, a.T * a.G);
     if (a.precision == 1) {
-        // the generalized gamma of free power runs the general per-node kernel
-        if (a.res == 2) k_forward<float, 2><<<grid, FWD_WARPS * 32, 0, st>>>(a);
-        else return launch_forward_mixed(a, st);
+        if (a.res != 2) return launch_forward_mixed(a, st);
+        // generalized gamma of free power: tiles of linear bins two bins per instruction, the tiles with
+        // log-spaced bins (the first of the histogram) by the general per-node kernel
+        const cudaError_t e = launch_forward_gg(a, st);
+        if (e != cudaSuccess) return e;
+        grid.x = (a.jlin_max + 31) / 32;
+        if (grid.x > 0) k_forward_gg_low<<<grid, FWD_WARPS * 32, 0, st>>>(a);
     } else {
         if (a.res == 0)      k_forward_gauss64<<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else if (a.res == 1) k_forward<double, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
@@ -1658,6 +1704,7 @@ cudaError_t launch_backward(const KArgs& a, cudaStream_t st) {
     if (a.pair) return launch_backward_pair(a, st);
     // the tuned mixed adjoint serves the Gaussian and gamma responses (with or without secondary observables)
     if (a.precision == 1 && a.res != 2) return launch_backward_mixed(a, st);
+    if (a.precision == 1 && !a.nsec) return launch_backward_gg(a, st);
     dim3 grid(a.nbtask, a.G, a.T);
     const int threads = a.bw_warps * 32;
     const size_t rs = a.precision == 1 ? sizeof(float) : sizeof(double);
