@@ -443,6 +443,7 @@ int finalize(gsn_ctx* c) {
     KArgs& a = c->base;
     a = KArgs{};
     a.D = c->D; a.S = c->S; a.K = c->K; a.P = c->P; a.NSLOT = NSLOT;
+    a.nsm = c->nsm;
     a.res = c->opt.resolution;
     a.precision = mixed ? 1 : 0;
     a.cut = c->opt.band_cut;

@@ -98,6 +98,7 @@ struct PairRec;
 struct KArgs {
     // problem
     int T, D, S, K, P, NSLOT, G, total_bins, nsplit, n_pulls;
+    int nsm;          // SMs of the device
     int res;          // 0 gauss, 1 gamma, 2 generalized gamma with a free power
     int precision;    // 0 fp64, 1 mixed
     double cut;       // band cut on the log-density
