@@ -1860,6 +1860,17 @@ int gsn_fit_rates_batch_dev(gsn_ctx* c, int n_toys, double* params_dev, const do
         if (a.response) {
             CUDA_TRY(c, cudaMemsetAsync(c->Mbuf.p, 0, (size_t)T * c->G * S * c->Jmax * sizeof(double), c->stream));
             if ((rc = launch(c, K_COLUMNS, a, launch_columns))) return rc;
+            // few toys: the column blocks of the per-species kernel among several CTAs (at most eight waves of
+            // two CTAs per SM), their sums apart in up to 2 GiB; without the memory one CTA adds them as it goes
+            const long long ctas = (long long)((c->Jmax + 255) / 256) * c->G * T * ((S + 15) / 16);
+            const size_t apart = (size_t)T * c->G * a.nblk * S * c->Jmax * sizeof(double);
+            if (ctas < 16LL * c->nsm && apart <= ((size_t)2 << 30) &&
+                !(c->opt.precision == GSN_FP64 && c->opt.resolution == GSN_RES_GAUSS) &&
+                ensure(c, c->sppart, apart) == GSN_OK) {
+                const int nq = (int)std::min<long long>((a.nblk + 3) / 4, (16LL * c->nsm + ctas - 1) / ctas);
+                a.sp_blocks = (a.nblk + nq - 1) / nq;
+                a.sp_part = (double*)c->sppart.p;
+            }
             if ((rc = launch(c, K_SPECIES, a, launch_species))) return rc;
         }
         RateArgs r{};

@@ -1401,13 +1401,13 @@ __global__ void __launch_bounds__(GF_THREADS) k_gradfinal(KArgs a) {
 // M[g][s][j] = sum_k R_jk S'_sk for species s in [sp_first, sp_first + sp_count)
 template <class R, int RES, int NG>
 DEV void species_loop(const KArgs& a, int t, int g, float xlo_w, float xhi_w, bool valid, bool is_zero,
-                      const R* nodes, R xc, double* accd, int nsp) {
+                      const R* nodes, R xc, double* accd, int nsp, int b0, int b1, double* part, long long bstride) {
     R del[NG], lam[NG], wt[NG];
     constexpr int NGM = sizeof(R) == 4 ? NGM_F : NGM_D;
 #pragma unroll
     for (int n = 0; n < NG; ++n) { del[n] = nodes[n]; lam[n] = nodes[NGM + n]; wt[n] = valid ? nodes[2 * NGM + n] : R(0); }
     const R* blk = reinterpret_cast<const R*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
-    for (int b = 0; b < a.nblk; ++b) {
+    for (int b = b0; b < b1; ++b) {
         if (blk[2 * b + 1] < (R)xlo_w || blk[2 * b] > (R)xhi_w) continue;
         R acc[16];
 #pragma unroll
@@ -1436,16 +1436,28 @@ DEV void species_loop(const KArgs& a, int t, int g, float xlo_w, float xhi_w, bo
                 }
             }
         }
+        if (part) {  // a block's sums of their own (k_species_sum adds them)
 #pragma unroll
-        for (int i = 0; i < 16; ++i) accd[i] += (double)acc[i];
+            for (int i = 0; i < 16; ++i)
+                if (i < nsp && valid) part[b * bstride + (long long)i * a.Jmax] = (double)acc[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) accd[i] += (double)acc[i];
+        }
     }
 }
 
-// grid (bin tiles, groups, toys x species chunks of 16): M[t][g][s][j] (toy stride a.mstride)
+// grid (bin tiles, groups, toys x species chunks of 16): M[t][g][s][j] (toy stride a.mstride).  Where that
+// leaves the GPU with less than a few waves (a.sp_blocks > 0), the column blocks of 256 are shared among
+// CTAs, sp_blocks each, and their sums, kept apart in sp_part [t][g][block][s][j], are added in the order
+// in which one CTA adds them: the same bits (64 toys of the FP64 two-dataset fit, 20000 columns: 146 -> 130 ms,
+// now bound by the FP64 pipe)
 template <class R, int RES>
 __global__ void __launch_bounds__(FWD_WARPS * 32) k_species(KArgs a) {
     const int tile = blockIdx.x, g = blockIdx.y;
-    const int nchunk = (a.sp_count + 15) / 16, t = blockIdx.z / nchunk, chunk = blockIdx.z % nchunk;
+    const int nchunk = (a.sp_count + 15) / 16, nq = a.sp_blocks > 0 ? (a.nblk + a.sp_blocks - 1) / a.sp_blocks : 1;
+    const int z = blockIdx.z / nq, q = blockIdx.z % nq, t = z / nchunk, chunk = z % nchunk;
+    const int b0 = q * a.sp_blocks, b1 = a.sp_blocks > 0 ? min(a.nblk, b0 + a.sp_blocks) : a.nblk;
     if (!tb_g_active(a, g)) return;  // no smeared species in the group
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int J = tb_g_bins(a, g);
@@ -1463,21 +1475,44 @@ __global__ void __launch_bounds__(FWD_WARPS * 32) k_species(KArgs a) {
     const int nsp = min(16, a.sp_count - chunk * 16);
     KArgs b = a;
     b.sp_first = a.sp_first + chunk * 16;
+    const long long bstride = (long long)a.S * a.Jmax;
+    double* part = a.sp_blocks > 0 ? a.sp_part + ((long long)t * a.G + g) * a.nblk * bstride + (long long)b.sp_first * a.Jmax + j : nullptr;
     double accd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) accd[i] = 0.0;
     if constexpr (sizeof(R) == 4) {
         const float* nodes = a.ntab_f + (long long)nb * 3 * NGM_F;
         const float xc = a.xc_f[nb];
-        if (low) species_loop<float, RES, NG_LOG_F>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, xc, accd, nsp);
-        else     species_loop<float, RES, NG_LIN_F>(b, t, g, xlo_w, xhi_w, valid, false, nodes, xc, accd, nsp);
+        if (low) species_loop<float, RES, NG_LOG_F>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, xc, accd, nsp, b0, b1, part, bstride);
+        else     species_loop<float, RES, NG_LIN_F>(b, t, g, xlo_w, xhi_w, valid, false, nodes, xc, accd, nsp, b0, b1, part, bstride);
     } else {
         const double* nodes = a.ntab_d + (long long)nb * 3 * NGM_D;
-        if (low) species_loop<double, RES, NG_LOG_D>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd, nsp);
-        else     species_loop<double, RES, NG_LIN_D>(b, t, g, xlo_w, xhi_w, valid, false, nodes, 0.0, accd, nsp);
+        if (low) species_loop<double, RES, NG_LOG_D>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd, nsp, b0, b1, part, bstride);
+        else     species_loop<double, RES, NG_LIN_D>(b, t, g, xlo_w, xhi_w, valid, false, nodes, 0.0, accd, nsp, b0, b1, part, bstride);
     }
-    if (valid)
+    if (valid && !part)
         for (int i = 0; i < nsp; ++i) a.Mbuf[(long long)t * a.mstride + ((long long)g * a.S + b.sp_first + i) * a.Jmax + j] = accd[i];
+}
+
+// grid (tiles of 256 bins, groups x species, toys): sum of the column blocks that k_species evaluated for
+// the bin's tile of 32, in order
+template <class R>
+__global__ void __launch_bounds__(256) k_species_sum(KArgs a) {
+    const int g = blockIdx.y / a.sp_count, s = a.sp_first + blockIdx.y % a.sp_count, t = blockIdx.z;
+    if (!tb_g_active(a, g)) return;
+    const int J = tb_g_bins(a, g), j = blockIdx.x * 256 + threadIdx.x;
+    if (j >= J) return;
+    const int j0 = j & ~31, jl = min(j0 + 31, J - 1);
+    const float xlo_w = (float)a.edges[tb_g_edge_off(a, g) + j0];
+    const float xhi_w = (float)a.edges[tb_g_edge_off(a, g) + jl + 1];
+    const R* blk = reinterpret_cast<const R*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
+    const double* part = a.sp_part + ((long long)t * a.G + g) * a.nblk * a.S * a.Jmax + (long long)s * a.Jmax + j;
+    double v = 0.0;
+    for (int b = 0; b < a.nblk; ++b) {
+        if (blk[2 * b + 1] < (R)xlo_w || blk[2 * b] > (R)xhi_w) continue;
+        v += part[(long long)b * a.S * a.Jmax];
+    }
+    a.Mbuf[(long long)t * a.mstride + ((long long)g * a.S + s) * a.Jmax + j] = v;
 }
 
 // FP64 Gaussian per-species path: exact erfc bin integrals (lanes <-> edges, 31 bins per warp)
@@ -1764,7 +1799,7 @@ cudaError_t launch_species(const KArgs& a, cudaStream_t st) {
         k_species_gauss64<<<grid, FWD_WARPS * 32, 0, st>>>(a);
         return cudaGetLastError();
     }
-    dim3 grid((a.Jmax + FWD_WARPS * 32 - 1) / (FWD_WARPS * 32), a.G, nchunk * a.T);
+    dim3 grid((a.Jmax + FWD_WARPS * 32 - 1) / (FWD_WARPS * 32), a.G, nchunk * a.T * (a.sp_blocks > 0 ? (a.nblk + a.sp_blocks - 1) / a.sp_blocks : 1));
     if (a.precision == 1) {
         if (a.res == 0)      k_species<float, 0><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else if (a.res == 1) k_species<float, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
@@ -1772,6 +1807,11 @@ cudaError_t launch_species(const KArgs& a, cudaStream_t st) {
     } else {
         if (a.res == 1) k_species<double, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else            k_species<double, 2><<<grid, FWD_WARPS * 32, 0, st>>>(a);
+    }
+    if (a.sp_blocks > 0) {
+        const dim3 gs((a.Jmax + 255) / 256, a.G * a.sp_count, a.T);
+        if (a.precision == 1) k_species_sum<float><<<gs, 256, 0, st>>>(a);
+        else k_species_sum<double><<<gs, 256, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
