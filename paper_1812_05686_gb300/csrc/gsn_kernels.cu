@@ -18,7 +18,10 @@
 //               through the slot map (section 2.2 parameter synchronisation)
 // Mixed precision: FP32 response build and contraction with double-float
 // column means, FP32 partial sums flushed to FP64 per column block, FP64
-// deviance and reductions.  FP64: everything in double.
+// reductions; the deviance's terms and w in FP32 pairs (48 bits) where their
+// range allows.  FP64: the response in FP32 pairs (gsn_pair64.cu) and the rest
+// in double; rate fits, secondary observables and problems whose pair buffers
+// do not fit the no-allocation scratch run the kernels here in double.
 #include "gsn_device.cuh"
 #include "gsn_ggamma.cuh"
 #include "gsn_pair.cuh"
@@ -68,7 +71,7 @@ template <class R> DEV void gamma_band(R c, R d, R& lo, R& hi) {
 // The band summary of 256 columns comes from one block of 256 threads, or, in launches of few columns, from
 // a cluster of four blocks of 64: the lowest columns of a gamma column take lgamma, digamma and exp in FP64,
 // and a whole block of them on one SM's FP64 pipe was the launch's longest chain (20000 columns of two
-// datasets: FP64 91 -> 59 us, mixed 47 -> 34 us; 1250 Gaussian columns 27 -> 21 us).
+// datasets: FP64 91 -> 59 us, mixed 47 -> 34 us; 2000 Gaussian columns 27 -> 21 us).
 constexpr int COLSMALL = 64;
 template <class R, int RES, bool FAST>
 __global__ void __launch_bounds__(COLBLK) k_columns(KArgs a) {
@@ -639,48 +642,45 @@ __global__ void __launch_bounds__(FWD_WARPS * 32) k_forward_gauss64(KArgs a) {
 }
 
 // ------------------------------------------------------------ deviance -----
-// bins [lo, hi) of edges ed[0..J] whose content of N(x; m, w) exceeds exp(-cut) of its peak density
-DEV void peak_bins(const double* ed, int J, double m, double w, double cut, int& lo, int& hi) {
-    const double z = sqrt(2.0 * cut);
-    const double xa = m - z * w, xb = m + z * w;
-    int l = 0, h = J;
-    while (l < h) { const int q = (l + h) >> 1; if (ed[q + 1] <= xa) l = q + 1; else h = q; }
-    lo = l;
-    l = 0; h = J;
-    while (l < h) { const int q = (l + h) >> 1; if (ed[q] < xb) l = q + 1; else h = q; }
-    hi = l;
-}
-
-// AnaPeak species of one dataset (at most MAXPK), with the bins their profile reaches;
-// r holds eps_d f_ds times the rate
+// AnaPeak species of one dataset (at most MAXPK): r holds eps_d f_ds times the rate; the profile, cut where
+// its density falls below exp(-cut) of its peak, reaches from xa to xb
 constexpr int MAXPK = 8;
 struct PeakInfo {
-    int s[MAXPK], lo[MAXPK], hi[MAXPK], n;
-    double r[MAXPK], m[MAXPK], w[MAXPK];
+    int s[MAXPK], n;
+    double r[MAXPK], m[MAXPK], w[MAXPK], xa[MAXPK], xb[MAXPK];
 };
 
+// whether a bin's edges reach into the profile of peak q
+DEV bool in_peak(const PeakInfo& pk, int q, double e0, double e1) { return !(e1 <= pk.xa[q]) && e0 < pk.xb[q]; }
+
 // Called by the whole block with the same d; returns the number of peaks (pk untouched when the
-// dataset has none, so no barrier is needed then).
+// dataset has none, so no barrier is needed then).  A lane per species: one thread that walked the species
+// and searched the edges for the profile's bins was a chain of some 50 dependent loads (deviance of one
+// point of two datasets: FP64 48 -> 39 us, mixed 35 -> 31 us).
 DEV int load_peaks(const KArgs& a, const double* prm, int d, PeakInfo& pk) {
     if (a.tb->ds_npk[d] == 0) return 0;
     __syncthreads();  // earlier readers of pk are done
-    if (threadIdx.x == 0) {
-        const double* ed = a.edges + tb_g_edge_off(a, tb_ds_group(a, d));
-        int np = 0;
-        for (int s = 0; s < a.S && np < MAXPK; ++s) {
-            const double f = a.rfac[d * a.S + s];
-            if (a.ft.sp_kind[s] != 2 || f == 0.0) continue;
-            const int pr = a.slot_map[d * a.NSLOT + s];
-            pk.s[np] = s;
-            pk.r[np] = pr >= 0 ? f * prm[pr] : 0.0;
-            pk.m[np] = prm[a.slot_map[d * a.NSLOT + a.S + 5 + 2 * s]];
-            pk.w[np] = prm[a.slot_map[d * a.NSLOT + a.S + 6 + 2 * s]];
-            int lo, hi;
-            peak_bins(ed, tb_ds_bins(a, d), pk.m[np], pk.w[np], a.cut, lo, hi);
-            pk.lo[np] = lo; pk.hi[np] = hi;
-            ++np;
+    if (threadIdx.x < 32) {
+        int n0 = 0;
+        for (int s0 = 0; s0 < a.S; s0 += 32) {
+            const int s = s0 + (int)threadIdx.x;
+            const double f = s < a.S ? a.rfac[d * a.S + s] : 0.0;
+            const bool has = s < a.S && a.ft.sp_kind[s] == 2 && f != 0.0;
+            const unsigned all = __ballot_sync(~0u, has);
+            const int np = n0 + __popc(all & ((1u << threadIdx.x) - 1u));
+            if (has && np < MAXPK) {
+                const int* slot = a.slot_map + d * a.NSLOT;
+                const int pr = slot[s];
+                const double m = prm[slot[a.S + 5 + 2 * s]], w = prm[slot[a.S + 6 + 2 * s]];
+                const double z = sqrt(2.0 * a.cut);
+                pk.s[np] = s;
+                pk.r[np] = pr >= 0 ? f * prm[pr] : 0.0;
+                pk.m[np] = m; pk.w[np] = w;
+                pk.xa[np] = m - z * w; pk.xb[np] = m + z * w;
+            }
+            n0 += __popc(all);
         }
-        pk.n = np;
+        if (threadIdx.x == 0) pk.n = min(n0, MAXPK);
     }
     __syncthreads();
     return pk.n;
@@ -767,7 +767,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
             if constexpr (sizeof(R) == 8) {
                 if (fhi > flo) {
                     __syncthreads();  // earlier readers of fs are done
-                    for (int i = threadIdx.x; i < (int)blockDim.x + 2 * FM; i += blockDim.x) {
+                    for (int i = threadIdx.x; i < min((int)blockDim.x, j1 - s0) + 2 * FM; i += blockDim.x) {
                         const int n = s0 - FM + i;
                         fs[i] = n >= flo && n < fhi ? sum_splits(frow + n, a.fext, a.nsplit) : 0.0;
                     }
@@ -788,7 +788,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                     }
                 }
                 for (int q = 0; q < npk; ++q) {
-                    if (j < pk.lo[q] || j >= pk.hi[q]) continue;
+                    if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
                     const double m = pk.m[q], wd = pk.w[q];
                     mu += pk.r[q] * ncdf_diff((ed[j] - m) / wd, (ed[j + 1] - m) / wd);
                 }
@@ -884,7 +884,8 @@ __global__ void __launch_bounds__(256) k_devfinal(KArgs a) {
                 const int pw = a.slot_map[d * a.NSLOT + a.S + 6 + 2 * s];
                 const double r = pk.r[q], m = pk.m[q], wd = pk.w[q];  // r = eps_d f_ds rate
                 double gr = 0.0, gm = 0.0, gw = 0.0;
-                for (int j = pk.lo[q] + threadIdx.x; j < pk.hi[q]; j += blockDim.x) {
+                for (int j = threadIdx.x; j < tb_ds_bins(a, d); j += blockDim.x) {
+                    if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
                     const double wj = a.precision == 1 ? (double)wf[off + j] : wd64[off + j];
                     if (wj == 0.0) continue;
                     const double z0 = (ed[j] - m) / wd, z1 = (ed[j + 1] - m) / wd;
@@ -932,10 +933,14 @@ __global__ void __launch_bounds__(256) k_devfinal(KArgs a) {
         }
         __syncthreads();  // gdir before thread 0 adds the pulls
     }
+    double nll = 0.0;
+    int flags = 0;
+    if (threadIdx.x < 32) {
+        for (int c = threadIdx.x; c < a.dev_chunks; c += 32) { nll += dp[pstride * c]; flags |= (int)dp[pstride * c + 1]; }
+        nll = warp_sum<double>(nll);
+        flags = __reduce_or_sync(~0u, flags);
+    }
     if (threadIdx.x == 0) {
-        double nll = 0.0;
-        int flags = 0;
-        for (int c = 0; c < a.dev_chunks; ++c) { nll += dp[pstride * c]; flags |= (int)dp[pstride * c + 1]; }
         // secondary-observable pieces (section 2.4): NLL, flags and slot gradients per dataset
         for (int i = 0; i < a.nsec; ++i) {
             const double* sp = a.secpart + ((long long)t * a.nsec + i) * (2 + a.NSLOT);
