@@ -1867,8 +1867,7 @@ int gsn_fit_rates_batch_dev(gsn_ctx* c, int n_toys, double* params_dev, const do
             if (ctas < 16LL * c->nsm && apart <= ((size_t)2 << 30) &&
                 !(c->opt.precision == GSN_FP64 && c->opt.resolution == GSN_RES_GAUSS) &&
                 ensure(c, c->sppart, apart) == GSN_OK) {
-                const int nq = (int)std::min<long long>((a.nblk + 3) / 4, (16LL * c->nsm + ctas - 1) / ctas);
-                a.sp_blocks = (a.nblk + nq - 1) / nq;
+                a.sp_parts = (int)std::min<long long>(a.nblk, (16LL * c->nsm + ctas - 1) / ctas);
                 a.sp_part = (double*)c->sppart.p;
             }
             if ((rc = launch(c, K_SPECIES, a, launch_species))) return rc;

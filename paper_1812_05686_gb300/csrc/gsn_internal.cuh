@@ -219,7 +219,7 @@ struct KArgs {
     float2* wfbuf;              // [T][fext] filtered weights
     const float2* Sp;           // [nbat 32][S padded to SPW] S' SPEC_SCALE (NULL: spectra the pairs do not hold)
     int sp_nsplit;              // batch splits of the per-species kernel in pairs
-    int sp_blocks;              // column blocks of 256 per CTA of the general per-species kernel (0: all)
+    int sp_parts;               // general per-species kernel: CTAs that share the column blocks (0: one, no sums apart)
     double* sp_part;            // pairs: [T][G][sp_nsplit][S][centres, bins][Jmax + FM]; general: [T][G][nblk][S][Jmax]
     // tensor-core per-species contraction
     int tc_nsplit;         // column ranges per bin tile

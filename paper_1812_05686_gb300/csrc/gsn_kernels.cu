@@ -1406,13 +1406,13 @@ __global__ void __launch_bounds__(GF_THREADS) k_gradfinal(KArgs a) {
 // M[g][s][j] = sum_k R_jk S'_sk for species s in [sp_first, sp_first + sp_count)
 template <class R, int RES, int NG>
 DEV void species_loop(const KArgs& a, int t, int g, float xlo_w, float xhi_w, bool valid, bool is_zero,
-                      const R* nodes, R xc, double* accd, int nsp, int b0, int b1, double* part, long long bstride) {
+                      const R* nodes, R xc, double* accd, int nsp, int b0, int bstep, double* part, long long bstride) {
     R del[NG], lam[NG], wt[NG];
     constexpr int NGM = sizeof(R) == 4 ? NGM_F : NGM_D;
 #pragma unroll
     for (int n = 0; n < NG; ++n) { del[n] = nodes[n]; lam[n] = nodes[NGM + n]; wt[n] = valid ? nodes[2 * NGM + n] : R(0); }
     const R* blk = reinterpret_cast<const R*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
-    for (int b = b0; b < b1; ++b) {
+    for (int b = b0; b < a.nblk; b += bstep) {
         if (blk[2 * b + 1] < (R)xlo_w || blk[2 * b] > (R)xhi_w) continue;
         R acc[16];
 #pragma unroll
@@ -1453,16 +1453,17 @@ DEV void species_loop(const KArgs& a, int t, int g, float xlo_w, float xhi_w, bo
 }
 
 // grid (bin tiles, groups, toys x species chunks of 16): M[t][g][s][j] (toy stride a.mstride).  Where that
-// leaves the GPU with less than a few waves (a.sp_blocks > 0), the column blocks of 256 are shared among
-// CTAs, sp_blocks each, and their sums, kept apart in sp_part [t][g][block][s][j], are added in the order
-// in which one CTA adds them: the same bits (64 toys of the FP64 two-dataset fit, 20000 columns: 146 -> 130 ms,
-// now bound by the FP64 pipe)
+// leaves the GPU with less than a few waves (a.sp_parts > 0), the column blocks of 256 are dealt in turn to
+// sp_parts CTAs, so that each of a CTA's warps keeps a share of its band; their sums, kept apart in sp_part
+// [t][g][block][s][j], are added in the order in which one CTA adds them: the same bits.  Calls of
+// two-dataset FP64 fits: 64 toys, 512 bins, 20000 columns 78.8 -> 63.6 ms; 10 toys, 1200, 14000 61.0 -> 23.4 ms;
+// 48 toys, 700, 8000, where one CTA per SM fits evenly, 40.2 -> 38.4 ms.  Runs of consecutive blocks instead left
+// most of a CTA's warps without a band to evaluate (73.1, 26.8 and 43.8 ms).
 template <class R, int RES>
 __global__ void __launch_bounds__(FWD_WARPS * 32) k_species(KArgs a) {
     const int tile = blockIdx.x, g = blockIdx.y;
-    const int nchunk = (a.sp_count + 15) / 16, nq = a.sp_blocks > 0 ? (a.nblk + a.sp_blocks - 1) / a.sp_blocks : 1;
-    const int z = blockIdx.z / nq, q = blockIdx.z % nq, t = z / nchunk, chunk = z % nchunk;
-    const int b0 = q * a.sp_blocks, b1 = a.sp_blocks > 0 ? min(a.nblk, b0 + a.sp_blocks) : a.nblk;
+    const int nchunk = (a.sp_count + 15) / 16, bstep = max(1, a.sp_parts);
+    const int z = blockIdx.z / bstep, b0 = blockIdx.z % bstep, t = z / nchunk, chunk = z % nchunk;
     if (!tb_g_active(a, g)) return;  // no smeared species in the group
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int J = tb_g_bins(a, g);
@@ -1481,19 +1482,19 @@ __global__ void __launch_bounds__(FWD_WARPS * 32) k_species(KArgs a) {
     KArgs b = a;
     b.sp_first = a.sp_first + chunk * 16;
     const long long bstride = (long long)a.S * a.Jmax;
-    double* part = a.sp_blocks > 0 ? a.sp_part + ((long long)t * a.G + g) * a.nblk * bstride + (long long)b.sp_first * a.Jmax + j : nullptr;
+    double* part = a.sp_parts > 0 ? a.sp_part + ((long long)t * a.G + g) * a.nblk * bstride + (long long)b.sp_first * a.Jmax + j : nullptr;
     double accd[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) accd[i] = 0.0;
     if constexpr (sizeof(R) == 4) {
         const float* nodes = a.ntab_f + (long long)nb * 3 * NGM_F;
         const float xc = a.xc_f[nb];
-        if (low) species_loop<float, RES, NG_LOG_F>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, xc, accd, nsp, b0, b1, part, bstride);
-        else     species_loop<float, RES, NG_LIN_F>(b, t, g, xlo_w, xhi_w, valid, false, nodes, xc, accd, nsp, b0, b1, part, bstride);
+        if (low) species_loop<float, RES, NG_LOG_F>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, xc, accd, nsp, b0, bstep, part, bstride);
+        else     species_loop<float, RES, NG_LIN_F>(b, t, g, xlo_w, xhi_w, valid, false, nodes, xc, accd, nsp, b0, bstep, part, bstride);
     } else {
         const double* nodes = a.ntab_d + (long long)nb * 3 * NGM_D;
-        if (low) species_loop<double, RES, NG_LOG_D>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd, nsp, b0, b1, part, bstride);
-        else     species_loop<double, RES, NG_LIN_D>(b, t, g, xlo_w, xhi_w, valid, false, nodes, 0.0, accd, nsp, b0, b1, part, bstride);
+        if (low) species_loop<double, RES, NG_LOG_D>(b, t, g, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd, nsp, b0, bstep, part, bstride);
+        else     species_loop<double, RES, NG_LIN_D>(b, t, g, xlo_w, xhi_w, valid, false, nodes, 0.0, accd, nsp, b0, bstep, part, bstride);
     }
     if (valid && !part)
         for (int i = 0; i < nsp; ++i) a.Mbuf[(long long)t * a.mstride + ((long long)g * a.S + b.sp_first + i) * a.Jmax + j] = accd[i];
@@ -1804,7 +1805,7 @@ cudaError_t launch_species(const KArgs& a, cudaStream_t st) {
         k_species_gauss64<<<grid, FWD_WARPS * 32, 0, st>>>(a);
         return cudaGetLastError();
     }
-    dim3 grid((a.Jmax + FWD_WARPS * 32 - 1) / (FWD_WARPS * 32), a.G, nchunk * a.T * (a.sp_blocks > 0 ? (a.nblk + a.sp_blocks - 1) / a.sp_blocks : 1));
+    dim3 grid((a.Jmax + FWD_WARPS * 32 - 1) / (FWD_WARPS * 32), a.G, nchunk * a.T * std::max(1, a.sp_parts));
     if (a.precision == 1) {
         if (a.res == 0)      k_species<float, 0><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else if (a.res == 1) k_species<float, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
@@ -1813,7 +1814,7 @@ cudaError_t launch_species(const KArgs& a, cudaStream_t st) {
         if (a.res == 1) k_species<double, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
         else            k_species<double, 2><<<grid, FWD_WARPS * 32, 0, st>>>(a);
     }
-    if (a.sp_blocks > 0) {
+    if (a.sp_parts > 0) {
         const dim3 gs((a.Jmax + 255) / 256, a.G * a.sp_count, a.T);
         if (a.precision == 1) k_species_sum<float><<<gs, 256, 0, st>>>(a);
         else k_species_sum<double><<<gs, 256, 0, st>>>(a);

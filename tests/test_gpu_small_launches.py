@@ -1,5 +1,5 @@
-"""Launches too small for the GPU split their columns over clusters and their column blocks over thread
-blocks; a batch large enough is evaluated without either.  Both add in the same order: the same bits."""
+"""Launches too small for the GPU split their columns over clusters and deal their column blocks to several
+thread blocks; a batch large enough is evaluated without either.  Both add in the same order: the same bits."""
 import numpy as np
 import pytest
 
@@ -8,7 +8,8 @@ from paper_1812_05686_gb300 import inputs as I
 pytestmark = pytest.mark.gpu
 
 
-# column blocks of 256: one, two with a remainder of one column, ten (three groups of four, the last short)
+# column blocks of 256: one, two (the second of one column), ten; dealt to as many thread blocks as there are
+# column blocks (3 toys), to fewer (700 toys: four) or to one (2500 toys)
 @pytest.mark.parametrize("precision", ["FP64", "MIXED"])
 @pytest.mark.parametrize("J,K,power", [(40, 250, 0), (33, 257, 0), (60, 2500, 0), (60, 2500, 1.3)])
 def test_small_and_large_fits_have_the_same_bits(J, K, power, precision):
@@ -29,11 +30,11 @@ def test_small_and_large_fits_have_the_same_bits(J, K, power, precision):
     wins = torch.tensor([[[0, J], [0, J]]] * T, dtype=torch.int32, device=dev)
     lo = np.where(free, 0.0, -np.inf)
     out = []
-    for n in (T, few):
+    for n in (T, 700, few):
         x = torch.tensor(np.repeat(w["theta0"][None], n, axis=0), device=dev)
         nll, iters, status = ctx.fit_rates_batch_dev(x, counts[:n].contiguous(), wins[:n].contiguous(), free, lo=lo)
         torch.cuda.synchronize(dev)
         out.append([v[:few].cpu().numpy() for v in (x, nll, iters, status)])
     assert np.all(np.isfinite(out[0][1]))
-    for a, b in zip(*out):
-        assert np.array_equal(a, b)
+    for a, b, c in zip(*out):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
