@@ -7,7 +7,7 @@ domain of 1 p.e. bins, 23 parameters, two pulls.  Toy t has Poisson counts
 drawn from the stored expected counts at theta0 (seed 1000 + t), its own
 parameter vector theta0 (1 + 0.01 N(0,1)) and a fit window of 600..1200 bins.
 One step = one NLL + gradient evaluation of every toy (column prologue,
-response build + contraction, FP64 deviance and reduction, adjoint, gradient
+response build + contraction, deviance and FP64 reduction, adjoint, gradient
 reduction) in the mixed-precision path; inputs resident in HBM.
 
 Under torchrun each rank evaluates its own T toys (weak scaling, no collective
@@ -503,7 +503,7 @@ def run_ours(args, rank, world, local_rank):
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
-                "vs_baseline": None, "dtype": "f32 (f64 deviance and reductions)", "data": "synthetic",
+                "vs_baseline": None, "dtype": "f32 (f64 reductions, deviance terms in f32 pairs)", "data": "synthetic",
                 "config": {"workload": (WORKLOAD if not gg else
                            WORKLOAD.replace("gamma response, 23 params",
                                             f"generalized-gamma response of free power p = {args.power:g}, 24 params"))
@@ -689,7 +689,7 @@ def run_multivariate(args):
     achieved = kunits / max(kn, 1) * FLOP_PER_PAIR[dom] / per_launch_s
     line = {"metric": "NLL+grad evals/sec (batched toys, 2-D multivariate workload) on 1 GB300", "value": value,
             "unit": UNIT, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
-            "higher_is_better": True, "dtype": "f32 (f64 deviance and reductions)", "data": "synthetic",
+            "higher_is_better": True, "dtype": "f32 (f64 reductions, deviance terms in f32 pairs)", "data": "synthetic",
             "config": {"workload": MV_WORKLOAD, "toys": T, "datasets": D, "precision": "mixed",
                        "plan": ctx.plan_info(min(T, 83), True)},
             "fp64_path": fp64, "status_nonzero_toys": int(torch.count_nonzero(status).item()),
@@ -706,7 +706,7 @@ TPL_WORKLOAD = ("template_like: Monte Carlo template fit, 2 datasets x 1000 bins
 
 
 def run_templates(args):
-    """Batched toys of a pure template fit: only the FP64 deviance stage runs (no response)."""
+    """Batched toys of a pure template fit: only the deviance stage runs (no response)."""
     import numpy as np
     import torch
 
@@ -753,17 +753,18 @@ def run_templates(args):
     prof = ctx.profile_read()
     ctx.profile(False)
     clk = clocks.stop()
-    # roofline of the deviance stage: FP64, 2 FMA per template and bin (mu and the rate gradient)
+    # roofline of the deviance stage: FP64, one FMA per template and bin (mu; the rate gradient's products
+    # are FP32 pairs)
     S = w["spectra"].shape[0]
     kms, kn, _ = prof["deviance"]
     per_launch_s = kms * 1e-3 / max(kn, 1)
     bins_per_launch = min(T, 4096) * D * nb
-    flops = bins_per_launch * 4.0 * S
+    flops = bins_per_launch * 2.0 * S
     dfma = gsn.peak_probe(gsn.GSN_PROBE_DFMA)
     hbm = bins_per_launch * (8 + 4)  # counts read, w written (FP32)
     line = {"metric": "NLL+grad evals/sec (batched toys, Monte Carlo template fit) on 1 GB300", "value": T / (ms * 1e-3),
             "unit": UNIT, "n_gpus": 1, "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms,
-            "higher_is_better": True, "dtype": "f64 (template contraction and deviance)", "data": "synthetic",
+            "higher_is_better": True, "dtype": "f64 (template contraction; deviance terms and rate gradients in f32 pairs)", "data": "synthetic",
             "config": {"workload": TPL_WORKLOAD, "toys": T},
             "status_nonzero_toys": int(torch.count_nonzero(status).item()),
             "roofline": {"bound": "alu (fp64)", "achieved": flops / per_launch_s / 1e12, "peak": 2 * dfma / 1e12,
@@ -852,7 +853,7 @@ def run_discovery(args):
     st = np.concatenate([s1.cpu().numpy(), s0.cpu().numpy()])
     line = {"metric": "profile-likelihood fits/sec (batched toys, discovery test) on 1 GB300", "value": 2 * T / dt,
             "unit": "fits/s", "n_gpus": 1, "ms_total": dt * 1e3, "higher_is_better": True,
-            "dtype": "f32 response, f64 deviance and minimiser state", "data": "synthetic",
+            "dtype": "f32 response, f64 sums and minimiser state", "data": "synthetic",
             "config": {"workload": WORKLOAD + "; every toy in its own window (600..1200 bins)", "toys": T,
                        "free": [w["param_names"][i] for i in np.nonzero(free)[0]], "signal": w["param_names"][sig],
                        "minimiser": ("projected Newton on the rates with the exact Hessian (response held), "

@@ -53,10 +53,12 @@ extern "C" {
 #define GSN_ERR_NOMEM            -6  /* device allocation failed */
 #define GSN_ERR_TIMEOUT          -7  /* a bounded wait inside a kernel gave up (results not written) */
 
-/* precision of the response build and contraction (the deviance and the
- * NLL reduction are FP64 in both modes) */
+/* precision of the response build and contraction (the NLL reduction is FP64
+ * in both modes).  GSN_FP64 evaluates the response in unevaluated pairs of
+ * FP32 numbers (48 bits) where that is as accurate as FP64 arithmetic with
+ * Gauss-Legendre nodes, and in FP64 elsewhere. */
 #define GSN_FP64                  0
-#define GSN_MIXED                 1  /* FP32 response + contraction, FP64 deviance */
+#define GSN_MIXED                 1  /* FP32 response + contraction; deviance terms FP64 or FP32 pairs */
 
 /* resolution shape (section 2.3) */
 #define GSN_RES_GAUSS             0
@@ -411,7 +413,7 @@ int gsn_plan_info(gsn_ctx* ctx, int n_toys, int grad, int* out5);
  * paper's method: measurement support for the roofline of each kernel. */
 #define GSN_K_COLUMNS    0   /* column prologue: means, resolution, band, T_dk */
 #define GSN_K_FORWARD    1   /* response build + contraction -> mu */
-#define GSN_K_DEVIANCE   2   /* FP64 deviance over bin ranges, w = 1 - n/mu */
+#define GSN_K_DEVIANCE   2   /* deviance over bin ranges, w = 1 - n/mu */
 #define GSN_K_BACKWARD   3   /* adjoint over the band */
 #define GSN_K_GRADFINAL  4   /* partial-gradient reduction and slot-map scatter */
 #define GSN_K_SPECIES    5   /* per-species contraction (gsn_eval, gsn_expected) */
