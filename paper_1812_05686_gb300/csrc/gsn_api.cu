@@ -636,7 +636,7 @@ int finalize(gsn_ctx* c) {
     }
     int rc;
     a.pair = (!mixed && c->sec.empty() && a.response) ? 1 : 0;
-    a.fconv = a.pair;
+    a.fconv = a.stray = a.pair;
     a.nbat = (c->K + 31) / 32;
     a.fext = c->total_bins + c->D * FM;
     if (a.pair && (rc = pair_tables(c, ntab_d, bcls))) return rc;
@@ -1633,16 +1633,25 @@ int gsn_eval(gsn_ctx* c, const double* params, double* nll) {
     a.Mbuf = (double*)c->Mbuf.p;  // the cached shapes (one parameter point)
     a.secRq = nullptr;            // the secondary pieces take their slice sums from them
     a.fconv = 0;                  // mu is complete
+    a.stray = a.pair ? 2 : 0;     // the column records may be another point's
     if ((rc = launch(c, K_MU, a, launch_mu_from_species))) return rc;
     if (a.nsec && (rc = launch(c, K_SPECIES, a, launch_secondary))) return rc;
-    if ((rc = launch(c, K_DEVIANCE, a, launch_deviance))) return rc;
-    if ((rc = launch(c, K_DEVFINAL, a, launch_devfinal))) return rc;
     double* hout = c->host + c->P;
-    CUDA_TRY(c, cudaMemcpyAsync(hout, c->point_b.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-    *nll = hout[0];
     int st;
-    std::memcpy(&st, hout + 1, sizeof st);
+    auto deviance = [&]() -> int {
+        int r;
+        if ((r = launch(c, K_DEVIANCE, a, launch_deviance)) || (r = launch(c, K_DEVFINAL, a, launch_devfinal))) return r;
+        CUDA_TRY(c, cudaMemcpyAsync(hout, c->point_b.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+        *nll = hout[0];
+        std::memcpy(&st, hout + 1, sizeof st);
+        return GSN_OK;
+    };
+    if ((rc = deviance())) return rc;
+    if (st == 1) {  // counts where the spectra end: the expectations there from this point's column records
+        a.stray = 1;
+        if ((rc = launch(c, K_COLUMNS, a, launch_columns)) || (rc = deviance())) return rc;
+    }
     if (!hit && (rc = species_status(c))) return rc;
     return status_message(c, st, 0);
 }
@@ -2018,7 +2027,7 @@ extern "C" int gsn_eval_grad_noalloc(gsn_ctx* c, const double* params_dev, doubl
     size_t off[NBUF], total;
     // FP64 in pairs where its records fit the array, else the FP64 kernels, which need less
     for (int pair = a.pair;; pair = 0) {
-        a.pair = a.fconv = pair;
+        a.pair = a.fconv = a.stray = pair;
         p = heuristic_plan(c, 1, pair != 0);
         p.nsub = 1;
         const PairSizes z = pair ? pair_sizes(c, 1, p) : PairSizes{0, 0, 0, 0, 0};

@@ -204,6 +204,8 @@ struct KArgs {
     // FP64 response in FP32 pairs (gsn_pair64.cu): tables, per-launch records and sums
     int pair;                   // the context's response kernels work in pairs
     int fconv;                  // the deviance adds the smooth columns' bin integrals from fbuf
+    int stray;                  // bins of counts far above their expectation (gsn_pair.cuh): 1 = the deviance takes
+                                // their expectation from the column records in FP64, 2 = it reports them (status 1)
     const float2* ex2tab;       // [1024] 2^(i/1024)
     const double* conv;         // [FM + 1] coefficients of the bin integral over bin centres
     const double* tref;         // [tile][4] reference point x_r, ln x_r, 1/x_r

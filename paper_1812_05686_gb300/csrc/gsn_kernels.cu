@@ -706,11 +706,40 @@ DEV double sum_splits(const double* p, long long stride, int n) {
     return (s0 + s1) + (s2 + s3);
 }
 
+// Response part of a stray bin's expectation (gsn_pair.cuh): the sum over the columns whose band reaches
+// the bin's tile of 32, as the FP64 kernels take it, by a whole warp (lanes <-> columns)
+template <int RES>
+DEV double stray_sum_res(const KArgs& a, int t, int d, int j) {
+    const int g = tb_ds_group(a, d), dd = a.tb->ds_in_group[d], lane = threadIdx.x & 31;
+    int wlo, whi;
+    toy_window_union(a, t, g, wlo, whi);
+    const double* ed = a.edges + tb_g_edge_off(a, g);
+    const int j0 = j & ~31;
+    const float xlo = (float)ed[max(j0, wlo)], xhi = (float)ed[min(j0 + 32, whi)];
+    const float4* bsum = a.batsum + ((long long)t * a.G + g) * a.nbat;
+    double v = 0.0;
+    for (int b0 = 0; b0 < a.nbat; b0 += 32) {
+        float4 bs = make_float4(INFINITY, -INFINITY, 0.f, 0.f);
+        if (b0 + lane < a.nbat) bs = bsum[b0 + lane];
+        for (unsigned m = __ballot_sync(0xffffffffu, !(bs.y < xlo || bs.x > xhi)); m; m &= m - 1) {
+            const int k = (b0 + __ffs(m) - 1) * 32 + lane;
+            if (k >= a.K) continue;
+            const double* c = colrec<double>(a, t, g, k);
+            if (c[F_TN0 + dd] == 0.0 || c[F_XMAX] < (double)xlo || c[F_XMIN] > (double)xhi) continue;
+            v = fma(native_value<RES>(a, t, g, k, c, j), c[F_TN0 + dd], v);
+        }
+    }
+    return warp_sum<double>(v);
+}
+static __device__ __noinline__ double stray_sum(const KArgs& a, int t, int d, int j) {
+    return a.res == 0 ? stray_sum_res<0>(a, t, d, j) : a.res == 1 ? stray_sum_res<1>(a, t, d, j) : stray_sum_res<2>(a, t, d, j);
+}
+
 // Stage 1 of the deviance, grid (T, dev_chunks): every block takes one contiguous range of the
 // concatenated bins of a toy, completes mu (split sum + AnaPeak profiles), writes
 // w = 1 - n/mu for the adjoint and the block's partial sum of the Eq. (LL) terms and status flags.
 template <class R>
-__global__ void __launch_bounds__(256) k_deviance(KArgs a) {
+__global__ void __launch_bounds__(256, 4) k_deviance(const __grid_constant__ KArgs a) {
     const int t = blockIdx.x, c = blockIdx.y;
     __shared__ double sh[32];
     __shared__ PeakInfo pk;
@@ -730,6 +759,7 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
     double part = 0.0;
     float ph = 0.f, pl = 0.f;   // the terms that pairs hold
     int bad_mu = 0, bad_fin = 0;
+    [[maybe_unused]] bool any_stray = false;
     for (int d = 0; d < a.D; ++d) {
         const int J = tb_ds_bins(a, d), off = tb_ds_off(a, d);
         const int j0 = max(0, b0 - off), j1 = min(J, b1 - off);
@@ -774,10 +804,21 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                     __syncthreads();
                 }
             }
-            if (j >= j1) continue;
+            const bool inw = j < j1 && j >= lo && j < hi;
             R w = 0;
-            if (j >= lo && j < hi) {
-                double mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
+            double mu = 0.0, n = 0.0;
+            // peaks and templates of a bin
+            auto direct = [&](double mu) {
+                for (int q = 0; q < npk; ++q) {
+                    if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
+                    const double m = pk.m[q], wd = pk.w[q];
+                    mu += pk.r[q] * ncdf_diff((ed[j] - m) / wd, (ed[j + 1] - m) / wd);
+                }
+                for (int q = 0; q < ntp; ++q) mu = fma(tcoef[q], a.tpl[toff[q] + j], mu);
+                return mu;
+            };
+            if (inw) {
+                mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
                 if constexpr (sizeof(R) == 8) {
                     const double* f = fs + threadIdx.x + FM;
                     if (fhi > flo && j >= ju && f[0] != 0.0) {
@@ -787,13 +828,22 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                         mu = fma(fma(a.conv[0], f[0], v), ed[j + 1] - ed[j], mu);
                     }
                 }
-                for (int q = 0; q < npk; ++q) {
-                    if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
-                    const double m = pk.m[q], wd = pk.w[q];
-                    mu += pk.r[q] * ncdf_diff((ed[j] - m) / wd, (ed[j + 1] - m) / wd);
+                mu = direct(mu);
+                n = cnt[off + j];
+            }
+            if constexpr (sizeof(R) == 8) {
+                if (a.stray && tb_ds_resp(a, d)) {
+                    const bool far = n > 0.0 && __double2hiint(n) - max(__double2hiint(mu), 0) > STRAY_RATIO;
+                    if (a.stray == 2) any_stray = any_stray || far;
+                    else
+                        for (unsigned m = __ballot_sync(0xffffffffu, far); m; m &= m - 1) {
+                            const int src = __ffs(m) - 1;
+                            const double v = stray_sum(a, t, d, s0 + (int)(threadIdx.x & ~31u) + src);
+                            if ((int)(threadIdx.x & 31) == src) mu = direct(v);
+                        }
                 }
-                for (int q = 0; q < ntp; ++q) mu = fma(tcoef[q], a.tpl[toff[q] + j], mu);
-                const double n = cnt[off + j];
+            }
+            if (inw) {
                 float th, tl;
                 if (n > 0.0 && poisson_term(mu, n, th, tl)) {
                     acc_pair(ph, pl, th, tl);
@@ -815,9 +865,10 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
                     if (!isfinite(mu)) bad_fin = 1;
                     part += term;
                     w = mu > 0.0 ? (R)(1.0 - n / mu) : R(0);
+                    if constexpr (sizeof(R) == 8) any_stray = any_stray || (a.stray == 1 && is_stray(w));
                 }
             }
-            wout[off + j] = w;
+            if (j < j1) wout[off + j] = w;
         }
         // template rate gradients: this block's share of sum_j w_j T_j (w as the adjoint reads it).  Mixed:
         // w is FP32, the products and sums are pairs (48 bits), a warp per template
@@ -852,9 +903,10 @@ __global__ void __launch_bounds__(256) k_deviance(KArgs a) {
     }
     const double sum = block_sum_d(part + join(ph, pl), sh);
     const int any_bad_mu = __syncthreads_or(bad_mu), any_bad_fin = __syncthreads_or(bad_fin);
+    const int stray_bins = sizeof(R) == 8 ? __syncthreads_or(any_stray) : 0;
     if (threadIdx.x == 0) {
         dp[0] = sum;
-        dp[1] = (double)(any_bad_mu | (any_bad_fin << 1));
+        dp[1] = (double)((any_bad_mu != 0) | ((any_bad_fin != 0) << 1) | ((stray_bins != 0) << 2));
     }
 }
 
@@ -963,6 +1015,7 @@ __global__ void __launch_bounds__(256) k_devfinal(KArgs a) {
         int st = 0;
         if (flags & 1) { st = -3; nll = INFINITY; }
         else if ((flags & 2) || !isfinite(nll)) st = -4;
+        if (a.stray == 2 && (flags & 4)) st = 1;   // the caller repeats the step with the column records
         a.nll[t] = nll;
         if (a.status) a.status[t] = st;
     }

@@ -18,6 +18,13 @@ constexpr double PAIR_TMIN = 1e-25, PAIR_TMAX = 1e30;
 constexpr double SPEC_SCALE = 1152921504606846976.0, SPEC_MIN = 1e-40;
 // a column with more than this share of its batch's weight is evaluated in FP64 beside the pairs
 constexpr float HEAVY_SHARE = 0.25f;
+// Stray bins: counts of 2^20 expectations or more, in the tails where a column's density leaves FP32's range
+// (a tile that a band touches reaches bins 20 sigma out, 1e-87 of the peak) and where w = 1 - n/mu may leave it too.
+// Their expectation and their part of the adjoint take the FP64 formulas.
+// STRAY_RATIO: the same bound on the difference of the high words of n and mu; STRAY_HI: high word of w = -2^20
+constexpr int STRAY_RATIO = 20 << 20;
+constexpr unsigned STRAY_HI = 0xC1300000u;
+DEV bool is_stray(double w) { return (unsigned)__double2hiint(w) >= STRAY_HI; }
 constexpr int SPW = 16;   // species per pass of the per-species kernel
 
 // One fine column.
@@ -33,6 +40,27 @@ struct __align__(16) PairRec {
     float2 T[MAXGDS];
 };
 static_assert(sizeof(PairRec) == 96, "three sectors");
+
+// FP64 bin value of one column (batches whose columns are too narrow for pairs, heavy columns, stray bins)
+template <int RES>
+DEV double native_value(const KArgs& a, int t, int g, int k, const double* c, int j) {
+    if constexpr (RES == 0) {
+        const double* ed = a.edges + tb_g_edge_off(a, g) + j;
+        return ncdf_diff((ed[0] - c[F_MUH]) * c[F_A], (ed[1] - c[F_MUH]) * c[F_A]);
+    } else {
+        const int nb = tb_g_node_off(a, g) + j;
+        const unsigned char cls = a.bclass[nb];
+        if (cls == BIN_ZERO) return zerorec<double>(a, t, g, k)[Z_P0];
+        const double* nd = a.ntab_d + (long long)nb * 3 * NGM_D;
+        const int NG = cls == BIN_LOG ? NG_LOG_D : NG_LIN_D;
+        double rho = 0.0;
+        for (int n = 0; n < NG; ++n) {
+            if constexpr (RES == 1) rho = fma(nd[2 * NGM_D + n], exp(fma(c[F_B], nd[NGM_D + n], fma(-c[F_C], nd[n], c[F_A]))), rho);
+            else rho = fma(nd[2 * NGM_D + n], exp(fma(c[F_B], nd[NGM_D + n], c[F_A]) - exp(c[F_KAPPA] * (nd[NGM_D + n] - c[F_C]))), rho);
+        }
+        return rho;
+    }
+}
 
 // ------------------------------------------------ arithmetic on pairs -----
 // TwoSum of a running pair (sh, sl) and p, error terms collected in sl

@@ -36,6 +36,8 @@
 // linear class); other bins and narrower columns take the Gauss-Legendre nodes of the bin with the
 // same evaluation (five, ten in the log-spaced bins, eight for the Gaussian), and columns below the
 // SQ_* limits, where the pairs' terms would cancel or the nodes miss a Gaussian, the FP64 formulas.
+// Bins that hold counts where the expectation is far below them (a million times and more) leave the
+// pairs as well (is_stray).
 // Classes are chosen per batch of 32 columns (the warp's) from the batch's smallest sigma.  A column
 // that outweighs its batch (a mono-energetic line) is evaluated in FP64 beside the pairs: the single
 // error of its pairs, 6e-15, would be the error of every bin it dominates.
@@ -84,8 +86,12 @@ DEV void pair_exp2(float s, float lo, int nb, const float2* __restrict__ tab, fl
 // of the size of g a.
 struct ColTerms { float2 E, g, P; int nb; };
 
-// density at the node (a, D); Gaussian: (ah, al) becomes x - mu and (Dh, Dl) its square
-template <int RES>
+// Density at the node (a, D); Gaussian: (ah, al) becomes x - mu and (Dh, Dl) its square.  The exponent is
+// held at a floor so that its bits do not wrap: 2^-125 of a Gaussian's peak, at most 2^-89 of the gamma
+// family's (nb is at most half above the exponent at x_r).  With CUT values at the floor are 0.  The forward and
+// the adjoint leave them, an instruction per value less: they enter a bin's expectation where it is above
+// 2^-20 of its counts only (is_stray), as 2^-69 of the counts or less.
+template <int RES, bool CUT = false>
 DEV void pair_density(const ColTerms& c, float& ah, float& al, float& Dh, float& Dl, const float2* __restrict__ tab, float& vh,
                       float& vl) {
     if constexpr (RES == 0) {
@@ -99,6 +105,7 @@ DEV void pair_density(const ColTerms& c, float& ah, float& al, float& Dh, float&
         float s, lo;
         mul_pair(c.P.x, c.P.y, Dh, Dl, s, lo);
         pair_exp2(fmaxf(s, -125.0f), lo, 0x3f800000, tab, vh, vl);
+        if (CUT && s < -125.0f) vh = vl = 0.f;
     } else {
         float p1, e1, p2, e2;
         mul_pair(c.g.x, c.g.y, ah, al, p1, e1);
@@ -108,7 +115,8 @@ DEV void pair_density(const ColTerms& c, float& ah, float& al, float& Dh, float&
         const float s2 = __fadd_rn(s1, p2), b2 = __fsub_rn(s2, s1);
         const float t2 = __fadd_rn(__fsub_rn(s1, __fsub_rn(s2, b2)), __fsub_rn(p2, b2));
         const float lo = __fadd_rn(__fadd_rn(c.E.y, __fadd_rn(e1, e2)), __fadd_rn(t1, t2));
-        pair_exp2(fmaxf(s2, -90.0f), lo, c.nb, tab, vh, vl);   // values that no sum sees are held at 2^-120
+        pair_exp2(fmaxf(s2, -90.0f), lo, c.nb, tab, vh, vl);
+        if (CUT && s2 < -90.0f) vh = vl = 0.f;
     }
 }
 
@@ -234,27 +242,6 @@ DEV double native_sums(const KArgs& a, int t, int g, int k, const double* c, int
         else { u[0] = fma(W, rho, u[0]); u[1] = fma(W, s1, u[1]); u[2] = fma(W, s2, u[2]); u[3] = fma(W, s3, u[3]); }
     }
     return rho;
-}
-
-// FP64 bin value of one column (the batches of class 0)
-template <int RES>
-DEV double native_value(const KArgs& a, int t, int g, int k, const double* c, int j) {
-    if constexpr (RES == 0) {
-        const double* ed = a.edges + tb_g_edge_off(a, g) + j;
-        return ncdf_diff((ed[0] - c[F_MUH]) * c[F_A], (ed[1] - c[F_MUH]) * c[F_A]);
-    } else {
-        const int nb = tb_g_node_off(a, g) + j;
-        const unsigned char cls = a.bclass[nb];
-        if (cls == BIN_ZERO) return zerorec<double>(a, t, g, k)[Z_P0];
-        const double* nd = a.ntab_d + (long long)nb * 3 * NGM_D;
-        const int NG = cls == BIN_LOG ? NG_LOG_D : NG_LIN_D;
-        double rho = 0.0;
-        for (int n = 0; n < NG; ++n) {
-            if constexpr (RES == 1) rho = fma(nd[2 * NGM_D + n], exp(fma(c[F_B], nd[NGM_D + n], fma(-c[F_C], nd[n], c[F_A]))), rho);
-            else rho = fma(nd[2 * NGM_D + n], exp(fma(c[F_B], nd[NGM_D + n], c[F_A]) - exp(c[F_KAPPA] * (nd[NGM_D + n] - c[F_C]))), rho);
-        }
-        return rho;
-    }
 }
 
 DEV void load_table(const KArgs& a, float2* tab) {
@@ -489,8 +476,9 @@ __global__ void __launch_bounds__(PW * 32, 2) k_forward_p(KArgs a) {
 }
 
 // ------------------------------------------------ filtered weights for the adjoint -----
-// wf_i = sum_m c_m h_(i - m) w_(i - m) over the bins >= ju (h: bin widths, equal up to rounding): the transpose of the bin integral of the smooth
-// columns, as FP32 pairs (grid: toys x blocks of nodes)
+// wf_i = sum_m c_m h_(i - m) w_(i - m) over the bins >= ju (h: bin widths, equal up to rounding): the
+// transpose of the bin integral of the smooth columns, as FP32 pairs, without the stray bins (grid: toys x
+// blocks of nodes)
 __global__ void __launch_bounds__(256) k_wfilter(KArgs a) {
     const int t = blockIdx.x, n = blockIdx.y * 256 + threadIdx.x;
     if (n >= a.fext) return;
@@ -504,7 +492,10 @@ __global__ void __launch_bounds__(256) k_wfilter(KArgs a) {
         const double* w = reinterpret_cast<const double*>(a.wbuf) + (long long)t * a.total_bins + tb_ds_off(a, d);
         for (int m = -FM; m <= FM; ++m) {
             const int j = i - m;
-            if (j >= ju && j < J) v = fma(a.conv[m < 0 ? -m : m] * w[j], ed[j + 1] - ed[j], v);
+            if (j >= ju && j < J) {
+                const double wj = w[j];
+                v = fma(a.conv[m < 0 ? -m : m] * (is_stray(wj) ? 0.0 : wj), ed[j + 1] - ed[j], v);
+            }
         }
     }
     a.wfbuf[(long long)t * a.fext + n] = split(v);
@@ -528,6 +519,9 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
     float4* sn = reinterpret_cast<float4*>(smem_raw + 8192) + warp * 32 * NV;
     double* su = reinterpret_cast<double*>(smem_raw + 8192 + sizeof(float4) * 32 * NV * W);   // [NDS][W*32]
     double* sresp = su + NDS * W * 32;                                                        // [W][NRESP]
+    // flags of the toy's deviance blocks (read beside the table, used where the tiles begin)
+    const double* dflag = a.devpart + (long long)t * a.dev_chunks * (2 + a.ntpl) + 1;
+    const double flag0 = lane < a.dev_chunks ? dflag[lane * (2 + a.ntpl)] : 0.0;
     load_table(a, tab);
     __syncthreads();
     const int cbw = task / a.bw_bsplit, bsp = task % a.bw_bsplit;
@@ -563,6 +557,9 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
         const int rlo = fhi > flo ? min(wlo, flo) : wlo, rhi = max(whi, fhi > flo ? fhi : whi);
         ja = max(ja, rlo); jb = min(jb, rhi);
         if (jb > ja) {
+            int flags = (int)flag0;
+            for (int q = lane + 32; q < a.dev_chunks; q += 32) flags |= (int)dflag[q * (2 + a.ntpl)];
+            const bool stray_toy = __any_sync(0xffffffffu, flags & 4);   // the deviance found stray bins
             const int t0 = ja >> 5, t1 = ((jb - 1) >> 5) + 1, ch = (t1 - t0 + a.bw_bsplit - 1) / a.bw_bsplit;
             const int ta = t0 + bsp * ch, tb = min(t1, ta + ch);
             const double pw = toy_power<RES>(a, t, g);
@@ -571,12 +568,14 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
 #pragma unroll
             for (int dd = 0; dd < NDS; ++dd) Tk[dd] = pc.T[dd];
             const double Nn = RES == 0 ? c[F_A] * INV_SQRT2PI : 1.0;
-            // weights of bin j, and their sum over the datasets with a column's T
-            auto weights = [&](int j, double* wj, double& Wj, const double* cc) {
+            // weights of bin j (those of stray bins, the others, or both), and their sum over the datasets
+            // with a column's T
+            auto weights = [&](int j, double* wj, double& Wj, const double* cc, bool plain, bool stray) {
 #pragma unroll
                 for (int dd = 0; dd < NDS; ++dd) {
-                    wj[dd] = dd < nds ? reinterpret_cast<const double*>(a.wbuf)[(long long)t * a.total_bins +
-                                                                                tb_ds_off(a, tb_g_ds(a, g, dd)) + j] : 0.0;
+                    const double w = dd < nds ? reinterpret_cast<const double*>(a.wbuf)[(long long)t * a.total_bins +
+                                                                                        tb_ds_off(a, tb_g_ds(a, g, dd)) + j] : 0.0;
+                    wj[dd] = (is_stray(w) ? stray : plain) ? w : 0.0;
                     Wj = fma(wj[dd], cc[F_TN0 + dd], Wj);
                 }
             };
@@ -618,7 +617,7 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
                     }
                     if (i >= max(lo, wlo) && i < min(min(hi, whi), cls == 2 ? ju : J)) {
                         double wj[NDS], Wj = 0.0;
-                        weights(i, wj, Wj, cc);
+                        weights(i, wj, Wj, cc, true, false);
                         const double rho = native_sums<RES>(a, t, g, kk, cc, i, Wj, hu);
 #pragma unroll
                         for (int dd = 0; dd < NDS; ++dd) hU[dd] = fma(wj[dd], rho, hU[dd]);
@@ -630,21 +629,30 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
                 for (int i = 0; i < (RES == 2 ? 5 : 2); ++i) { const double v = warp_sum<double>(hu[i]); if (lane == src) u[i] = v; }
             }
             const bool mine = !(hm >> lane & 1);   // the lane's column takes the pairs' sums
-            for (int tile = ta; tile < tb; ++tile) {
-                const int lo = max(ja, tile * 32), hi = min(jb, tile * 32 + 32);   // the band's bins in the tile
-                const int mlo = max(lo, wlo), mhi = min(min(hi, whi), J);
-                if (cls == 0) {
-                    // FP64 formulas, bin by bin
-                    for (int j = mlo; j < mhi; ++j) {
-                        ++nvisit;
+            // FP64 formulas, bin by bin: the band's bins of columns that the pairs do not take, and the tiles'
+            // stray bins for the columns that entered their expectation (stray_sum)
+            if (cls == 0 || stray_toy)
+                for (int tile = ta; tile < tb; ++tile) {
+                    const int mlo = max(max(ja, tile * 32), wlo), mhi = min(min(min(jb, tile * 32 + 32), whi), J);
+                    const int a0 = stray_toy ? max(tile * 32, wlo) : mlo, a1 = stray_toy ? min(min(tile * 32 + 32, whi), J) : mhi;
+                    const bool reach = stray_toy && !(c[F_XMAX] < (double)(float)ed[a0] || c[F_XMIN] > (double)(float)ed[a1]);
+                    for (int j = a0; j < a1; ++j) {
+                        const bool plain = cls == 0 && j >= mlo && j < mhi;
+                        nvisit += plain;
                         double wj[NDS], Wj = 0.0;
-                        weights(j, wj, Wj, c);
+                        weights(j, wj, Wj, c, plain, reach);
+                        bool any = false;
+#pragma unroll
+                        for (int dd = 0; dd < NDS; ++dd) any = any || wj[dd] != 0.0;
+                        if (!any) continue;
                         const double rho = native_sums<RES>(a, t, g, kval ? k : a.K - 1, c, j, Wj, u);
 #pragma unroll
                         for (int dd = 0; dd < NDS; ++dd) U0[dd] = fma(wj[dd], rho, U0[dd]);
                     }
-                    continue;
                 }
+            for (int tile = cls == 0 ? tb : ta; tile < tb; ++tile) {
+                const int lo = max(ja, tile * 32), hi = min(jb, tile * 32 + 32);   // the band's bins in the tile
+                const int mlo = max(lo, wlo), mhi = min(min(hi, whi), J);
                 const TileRef tr = tile_ref(a, g, tile);
                 double dl = 0.0, y = 0.0;
                 const ColTerms ct = column_terms<RES>(pc, tr, pw, dl, y);
@@ -737,8 +745,11 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
 #pragma unroll
                             for (int dd = 0; dd < NDS; ++dd)
                                 if (dd < nds)
-                                    wv[dd] = split(wt * reinterpret_cast<const double*>(a.wbuf)[(long long)t * a.total_bins +
-                                                                                               tb_ds_off(a, tb_g_ds(a, g, dd)) + jj]);
+                                {
+                                    const double w = reinterpret_cast<const double*>(a.wbuf)[(long long)t * a.total_bins +
+                                                                                             tb_ds_off(a, tb_g_ds(a, g, dd)) + jj];
+                                    wv[dd] = split(is_stray(w) ? 0.0 : wt * w);
+                                }
                         }
                         __syncwarp();
                         sn[lane * NV] = s;
@@ -750,7 +761,7 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
                     nvisit += nbin;
                     if (RES >= 1 && mlo == 0 && tb_g_zero(a, g) && mine) {
                         double wj[NDS], Wj = 0.0;
-                        weights(0, wj, Wj, c);
+                        weights(0, wj, Wj, c, true, false);
                         const double rho = native_sums<RES>(a, t, g, kval ? k : a.K - 1, c, 0, Wj, u);
 #pragma unroll
                         for (int dd = 0; dd < NDS; ++dd) U0[dd] = fma(wj[dd], rho, U0[dd]);
@@ -1009,7 +1020,7 @@ __global__ void __launch_bounds__(SPB * 32, 4) k_species_p(KArgs a) {
                 if (pass == 0) {
                     for (int ci = 0; ci < 32; ++ci) {
                         float xh = ah, xl = al, yh = Dh, yl = Dl, vh, vl;
-                        pair_density<RES>(terms(ci), xh, xl, yh, yl, tab, vh, vl);
+                        pair_density<RES, true>(terms(ci), xh, xl, yh, yl, tab, vh, vl);
                         add(ci, vh, vl);
                     }
                 } else {
@@ -1034,7 +1045,7 @@ __global__ void __launch_bounds__(SPB * 32, 4) k_species_p(KArgs a) {
                                 float2 qa = sq[(n * 3) * 32], qd = sq[(n * 3 + 1) * 32];
                                 const float2 qw = sq[(n * 3 + 2) * 32];
                                 float vh, vl, p, e;
-                                pair_density<RES>(c, qa.x, qa.y, qd.x, qd.y, tab, vh, vl);
+                                pair_density<RES, true>(c, qa.x, qa.y, qd.x, qd.y, tab, vh, vl);
                                 mul_pair(vh, vl, qw.x, qw.y, p, e);
                                 acc_pair(uh, ul, p, e);
                             }
