@@ -1845,6 +1845,7 @@ int gsn_fit_rates_batch_dev(gsn_ctx* c, int n_toys, double* params_dev, const do
     if ((rc = ensure(c, c->rfit_cfg, cfg.size() * sizeof(double) + icfg.size() * sizeof(int)))) return rc;
     const size_t nb = (size_t)T0 * c->total_bins;
     if ((rc = ensure(c, c->rfit_ws, nb * ((size_t)std::max(nf, 1) + 4) * sizeof(double)))) return rc;
+    c->cache_valid = false;   // the toys' shapes take the place of the cached point's
     if ((rc = ensure(c, c->Mbuf, (size_t)T0 * c->G * S * c->Jmax * sizeof(double)))) return rc;
     double* cf = (double*)c->rfit_cfg.p;
     int* ic = (int*)(cf + cfg.size());
