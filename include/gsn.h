@@ -54,9 +54,10 @@ extern "C" {
 #define GSN_ERR_TIMEOUT          -7  /* a bounded wait inside a kernel gave up (results not written) */
 
 /* precision of the response build and contraction (the NLL reduction is FP64
- * in both modes).  GSN_FP64 evaluates the response in unevaluated pairs of
- * FP32 numbers (48 bits) where that is as accurate as FP64 arithmetic with
- * Gauss-Legendre nodes, and in FP64 elsewhere. */
+ * in both modes; terms that FP32 pairs hold enter it in sums of at most 16).
+ * GSN_FP64 evaluates the response in unevaluated pairs of FP32 numbers (48 bits)
+ * where that is as accurate as FP64 arithmetic with Gauss-Legendre nodes, and in
+ * FP64 elsewhere. */
 #define GSN_FP64                  0
 #define GSN_MIXED                 1  /* FP32 response + contraction; deviance terms FP64 or FP32 pairs */
 

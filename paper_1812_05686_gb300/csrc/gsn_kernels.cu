@@ -757,7 +757,6 @@ __global__ void __launch_bounds__(256, 4) k_deviance(const __grid_constant__ KAr
     const long long sstride = a.total_bins;
     const double* mrow = a.mubuf + (long long)t * a.nrow * a.total_bins;
     double part = 0.0;
-    float ph = 0.f, pl = 0.f;   // the terms that pairs hold
     int bad_mu = 0, bad_fin = 0;
     [[maybe_unused]] bool any_stray = false;
     for (int d = 0; d < a.D; ++d) {
@@ -792,86 +791,92 @@ __global__ void __launch_bounds__(256, 4) k_deviance(const __grid_constant__ KAr
                 frow = a.fbuf + (long long)t * a.nsplit * a.fext + off + d * FM;
             }
         }
-        for (int s0 = j0; s0 < j1; s0 += blockDim.x) {
-            const int j = s0 + threadIdx.x;
-            if constexpr (sizeof(R) == 8) {
-                if (fhi > flo) {
-                    __syncthreads();  // earlier readers of fs are done
-                    for (int i = threadIdx.x; i < min((int)blockDim.x, j1 - s0) + 2 * FM; i += blockDim.x) {
-                        const int n = s0 - FM + i;
-                        fs[i] = n >= flo && n < fhi ? sum_splits(frow + n, a.fext, a.nsplit) : 0.0;
-                    }
-                    __syncthreads();
-                }
-            }
-            const bool inw = j < j1 && j >= lo && j < hi;
-            R w = 0;
-            double mu = 0.0, n = 0.0;
-            // peaks and templates of a bin
-            auto direct = [&](double mu) {
-                for (int q = 0; q < npk; ++q) {
-                    if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
-                    const double m = pk.m[q], wd = pk.w[q];
-                    mu += pk.r[q] * ncdf_diff((ed[j] - m) / wd, (ed[j + 1] - m) / wd);
-                }
-                for (int q = 0; q < ntp; ++q) mu = fma(tcoef[q], a.tpl[toff[q] + j], mu);
-                return mu;
-            };
-            if (inw) {
-                mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
+        // the terms that pairs hold, up to sixteen per thread: a pair that is never renormalised loses bits as the
+        // square of its terms (2000 equal ones: 3e-10), sixteen are good to 4e-14
+        for (int sa = j0; sa < j1; sa += 16 * blockDim.x) {
+            float ph = 0.f, pl = 0.f;
+            for (int s0 = sa; s0 < min(j1, sa + 16 * (int)blockDim.x); s0 += blockDim.x) {
+                const int j = s0 + threadIdx.x;
                 if constexpr (sizeof(R) == 8) {
-                    const double* f = fs + threadIdx.x + FM;
-                    if (fhi > flo && j >= ju && f[0] != 0.0) {
-                        double v = 0.0;
-#pragma unroll
-                        for (int m = FM; m > 0; --m) v = fma(a.conv[m], f[-m] + f[m], v);
-                        mu = fma(fma(a.conv[0], f[0], v), ed[j + 1] - ed[j], mu);
-                    }
-                }
-                mu = direct(mu);
-                n = cnt[off + j];
-            }
-            if constexpr (sizeof(R) == 8) {
-                if (a.stray && tb_ds_resp(a, d)) {
-                    const bool far = n > 0.0 && __double2hiint(n) - max(__double2hiint(mu), 0) > STRAY_RATIO;
-                    if (a.stray == 2) any_stray = any_stray || far;
-                    else
-                        for (unsigned m = __ballot_sync(0xffffffffu, far); m; m &= m - 1) {
-                            const int src = __ffs(m) - 1;
-                            const double v = stray_sum(a, t, d, s0 + (int)(threadIdx.x & ~31u) + src);
-                            if ((int)(threadIdx.x & 31) == src) mu = direct(v);
+                    if (fhi > flo) {
+                        __syncthreads();  // earlier readers of fs are done
+                        for (int i = threadIdx.x; i < min((int)blockDim.x, j1 - s0) + 2 * FM; i += blockDim.x) {
+                            const int n = s0 - FM + i;
+                            fs[i] = n >= flo && n < fhi ? sum_splits(frow + n, a.fext, a.nsplit) : 0.0;
                         }
+                        __syncthreads();
+                    }
                 }
-            }
-            if (inw) {
-                float th, tl;
-                if (n > 0.0 && poisson_term(mu, n, th, tl)) {
-                    acc_pair(ph, pl, th, tl);
-                    if constexpr (sizeof(R) == 4) {
-                        // w = (mu - n) / mu, the FP32 value the adjoint reads
-                        const float2 e = split(n - mu), m = split(mu);
-                        float q, qe;
-                        div_pair(-e.x, -e.y, m.x, m.y, q, qe);
-                        w = q + qe;
+                const bool inw = j < j1 && j >= lo && j < hi;
+                R w = 0;
+                double mu = 0.0, n = 0.0;
+                // peaks and templates of a bin
+                auto direct = [&](double mu) {
+                    for (int q = 0; q < npk; ++q) {
+                        if (!in_peak(pk, q, ed[j], ed[j + 1])) continue;
+                        const double m = pk.m[q], wd = pk.w[q];
+                        mu += pk.r[q] * ncdf_diff((ed[j] - m) / wd, (ed[j + 1] - m) / wd);
+                    }
+                    for (int q = 0; q < ntp; ++q) mu = fma(tcoef[q], a.tpl[toff[q] + j], mu);
+                    return mu;
+                };
+                if (inw) {
+                    mu = tb_ds_resp(a, d) ? sum_splits(mrow + off + j, sstride, a.nrow) : 0.0;
+                    if constexpr (sizeof(R) == 8) {
+                        const double* f = fs + threadIdx.x + FM;
+                        if (fhi > flo && j >= ju && f[0] != 0.0) {
+                            double v = 0.0;
+    #pragma unroll
+                            for (int m = FM; m > 0; --m) v = fma(a.conv[m], f[-m] + f[m], v);
+                            mu = fma(fma(a.conv[0], f[0], v), ed[j + 1] - ed[j], mu);
+                        }
+                    }
+                    mu = direct(mu);
+                    n = cnt[off + j];
+                }
+                if constexpr (sizeof(R) == 8) {
+                    if (a.stray && tb_ds_resp(a, d)) {
+                        const bool far = n > 0.0 && __double2hiint(n) - max(__double2hiint(mu), 0) > STRAY_RATIO;
+                        if (a.stray == 2) any_stray = any_stray || far;
+                        else
+                            for (unsigned m = __ballot_sync(0xffffffffu, far); m; m &= m - 1) {
+                                const int src = __ffs(m) - 1;
+                                const double v = stray_sum(a, t, d, s0 + (int)(threadIdx.x & ~31u) + src);
+                                if ((int)(threadIdx.x & 31) == src) mu = direct(v);
+                            }
+                    }
+                }
+                if (inw) {
+                    float th, tl;
+                    if (n > 0.0 && poisson_term(mu, n, th, tl)) {
+                        acc_pair(ph, pl, th, tl);
+                        if constexpr (sizeof(R) == 4) {
+                            // w = (mu - n) / mu, the FP32 value the adjoint reads
+                            const float2 e = split(n - mu), m = split(mu);
+                            float q, qe;
+                            div_pair(-e.x, -e.y, m.x, m.y, q, qe);
+                            w = q + qe;
+                        } else {
+                            w = 1.0 - n / mu;
+                        }
                     } else {
-                        w = 1.0 - n / mu;
+                        double term = mu;
+                        if (n > 0.0) {
+                            if (!(mu > 0.0)) { bad_mu = 1; term = INFINITY; }
+                            else term = mu - n + n * log(n / mu);
+                        }
+                        if (!isfinite(mu)) bad_fin = 1;
+                        part += term;
+                        w = mu > 0.0 ? (R)(1.0 - n / mu) : R(0);
+                        if constexpr (sizeof(R) == 8) any_stray = any_stray || (a.stray == 1 && is_stray(w));
                     }
-                } else {
-                    double term = mu;
-                    if (n > 0.0) {
-                        if (!(mu > 0.0)) { bad_mu = 1; term = INFINITY; }
-                        else term = mu - n + n * log(n / mu);
-                    }
-                    if (!isfinite(mu)) bad_fin = 1;
-                    part += term;
-                    w = mu > 0.0 ? (R)(1.0 - n / mu) : R(0);
-                    if constexpr (sizeof(R) == 8) any_stray = any_stray || (a.stray == 1 && is_stray(w));
                 }
+                if (j < j1) wout[off + j] = w;
             }
-            if (j < j1) wout[off + j] = w;
+            part += join(ph, pl);
         }
         // template rate gradients: this block's share of sum_j w_j T_j (w as the adjoint reads it).  Mixed:
-        // w is FP32, the products and sums are pairs (48 bits), a warp per template
+        // w is FP32 (6e-8), the products and sums are pairs, a warp per template
         if (sizeof(R) == 4 && ntp > 0) {
             __syncthreads();  // w of every thread
             const int ja = max(j0, lo), jb = min(j1, hi);
@@ -901,7 +906,7 @@ __global__ void __launch_bounds__(256, 4) k_deviance(const __grid_constant__ KAr
             if (threadIdx.x == 0) dp[2 + a.tb->ds_tpl0[d] + q] = gpart;
         }
     }
-    const double sum = block_sum_d(part + join(ph, pl), sh);
+    const double sum = block_sum_d(part, sh);
     const int any_bad_mu = __syncthreads_or(bad_mu), any_bad_fin = __syncthreads_or(bad_fin);
     const int stray_bins = sizeof(R) == 8 ? __syncthreads_or(any_stray) : 0;
     if (threadIdx.x == 0) {

@@ -811,17 +811,24 @@ __global__ void __launch_bounds__(256, 2) k_backward_p(KArgs a) {
                         u[3] = fma(y, fma(l, yb, M[1] + pw * M[3] + M[4]), u[3]);
                     }
                 }
-            }
-            // the pairs' part of the column (class 0 and the heavy columns have filled U0 and u)
-            if (mine) {
+                // every eight tiles the pairs' sums go to the column's FP64 sums (class 0 and the heavy columns have
+                // theirs there): a pair that is never renormalised loses bits as the square of its terms
+                if (((tile - ta) & 7) == 7 || tile + 1 == tb) {
+                    if (mine) {
 #pragma unroll
-                for (int dd = 0; dd < NDS; ++dd) U0[dd] = fma(Nn, join(Uh[dd], Ul[dd]), U0[dd]);
-                if constexpr (RES == 0) {
-                    u[0] = fma(c[F_A], join(Sh[1], Sl[1]), u[0]);
-                    u[1] += fma(c[F_A] * c[F_A], join(Sh[2], Sl[2]), -join(Sh[0], Sl[0]));
-                } else if constexpr (RES == 1) {
-                    u[0] += join(Sh[0], Sl[0]);
-                    u[1] += join(Sh[1], Sl[1]);
+                        for (int dd = 0; dd < NDS; ++dd) U0[dd] = fma(Nn, join(Uh[dd], Ul[dd]), U0[dd]);
+                        if constexpr (RES == 0) {
+                            u[0] = fma(c[F_A], join(Sh[1], Sl[1]), u[0]);
+                            u[1] += fma(c[F_A] * c[F_A], join(Sh[2], Sl[2]), -join(Sh[0], Sl[0]));
+                        } else if constexpr (RES == 1) {
+                            u[0] += join(Sh[0], Sl[0]);
+                            u[1] += join(Sh[1], Sl[1]);
+                        }
+                    }
+#pragma unroll
+                    for (int dd = 0; dd < NDS; ++dd) Uh[dd] = Ul[dd] = 0.f;
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) Sh[i] = Sl[i] = 0.f;
                 }
             }
         }
