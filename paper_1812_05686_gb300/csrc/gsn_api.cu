@@ -76,6 +76,7 @@ struct gsn_ctx {
     Buf zerobuf;             // bin-at-zero records [T][G][K][NFZ] (gamma-family responses)
     Buf colbuf, colbuf2, blkbuf, mubuf, wbuf, partbuf, gdirect, devbuf, params, counts_b, win_b, nll_b, grad_b, status_b, Mbuf,
         outbuf;
+    int toy_cap = 1 << 30;               // toys per launch that the device's memory held (batch_device)
     unsigned long long scratch_gen = 0;  // bumped whenever a buffer is (re)allocated
     // launch plans chosen by the autotuner, per (toys in a launch, gradient wanted)
     struct PlanRec { int nsplit, nsub, ntile, bw_warps, bw_bsplit, nbtask, dev_chunks; };
@@ -431,6 +432,7 @@ int finalize(gsn_ctx* c) {
         return fail(c, GSN_ERR_STATE, "gsn_set_data, gsn_set_species and gsn_set_params must all be called");
     if (c->stream) cudaStreamSynchronize(c->stream);
     drop_graphs(c);
+    c->toy_cap = 1 << 30;
     c->tuned.clear();
     free_owned(c);
     c->cache_valid = false;
@@ -790,6 +792,18 @@ int reserve(gsn_ctx* c, int T, const Plan& p, bool pair) {
     return GSN_OK;
 }
 
+// give back what reserve() allocated
+void release_scratch(gsn_ctx* c) {
+    drop_graphs(c);
+    for (Buf* b : {&c->colbuf, &c->zerobuf, &c->colbuf2, &c->blkbuf, &c->segbuf, &c->mubuf, &c->wbuf, &c->partbuf, &c->gdirect,
+                   &c->devbuf, &c->pairbuf, &c->batbuf, &c->fbuf, &c->wfbuf, &c->hvybuf, &c->secRq_b, &c->secN_b, &c->secV_b,
+                   &c->secW_b, &c->secpart_b, &c->secU_b}) {
+        if (b->p) cudaFree(b->p);
+        *b = Buf{};
+    }
+    ++c->scratch_gen;
+}
+
 // fill the plan and scratch fields of a (buffers reserved for at least T toys under p)
 void fill(gsn_ctx* c, int T, const Plan& p, KArgs& a) {
     a.work = nullptr;
@@ -1051,17 +1065,10 @@ int check_params_host(gsn_ctx* c, const double* params) {
     return GSN_OK;
 }
 
-// batched step on device pointers; T toys, chunked by max_toys_per_launch
-int batch_device(gsn_ctx* c, int n_toys, const double* params, const double* counts, const int* win,
+// batched step on device pointers, chunk toys per launch
+int batch_chunks(gsn_ctx* c, int chunk, int n_toys, const double* params, const double* counts, const int* win,
                  double* nll, double* grad, int* status) {
     int rc;
-    if ((rc = finalize(c))) return rc;
-    // toys per launch: the option, the grid limit of the forward (toys x groups <= 65535) and a
-    // 32 GiB bound on the column records (16 words per toy, group and fine column)
-    const size_t rec = (size_t)c->G * c->K * NFP * (c->opt.precision == GSN_MIXED ? sizeof(float) : sizeof(double));
-    const long long mem_cap = std::max<long long>(1, (long long)((size_t)32 << 30) / (long long)std::max<size_t>(rec, 1));
-    const int chunk = (int)std::max<long long>(1, std::min<long long>({(long long)c->opt.max_toys_per_launch,
-                                                                        65535LL / std::max(1, c->G), mem_cap}));
     const bool g = grad != nullptr;
     std::vector<KArgs> args;
     std::vector<Plan> plans;
@@ -1096,6 +1103,32 @@ int batch_device(gsn_ctx* c, int n_toys, const double* params, const double* cou
         }
         return (int)GSN_OK;
     });
+}
+
+// batched step on device pointers, chunked by max_toys_per_launch and by memory
+int batch_device(gsn_ctx* c, int n_toys, const double* params, const double* counts, const int* win,
+                 double* nll, double* grad, int* status) {
+    int rc;
+    if ((rc = finalize(c))) return rc;
+    // toys per launch: the option, the grid limit of the forward (toys x groups <= 65535) and a
+    // 32 GiB bound on the column records (16 words per toy, group and fine column; FP64 in pairs: their
+    // records, summaries and sums too)
+    size_t rec = (size_t)c->G * c->K * NFP * (c->opt.precision == GSN_MIXED ? sizeof(float) : sizeof(double));
+    if (c->base.pair) {
+        const PairSizes z = pair_sizes(c, 1, plan_with(c, 1, 1, 8, 1));
+        rec += z.rec + z.bat + z.f + z.wf + z.heavy;
+    }
+    const long long mem_cap = std::max<long long>(1, (long long)((size_t)32 << 30) / (long long)std::max<size_t>(rec, 1));
+    int chunk = (int)std::max<long long>(1, std::min<long long>({(long long)c->opt.max_toys_per_launch, 65535LL / std::max(1, c->G),
+                                                                  mem_cap, (long long)c->toy_cap}));
+    for (;;) {
+        rc = batch_chunks(c, chunk, n_toys, params, counts, win, nll, grad, status);
+        if (rc != GSN_ERR_NOMEM || chunk == 1 || stream_capturing(c)) return rc;
+        // the device has less left than a launch of this many toys takes (nothing is enqueued yet): half as
+        // many, and no more in later calls on this problem
+        release_scratch(c);
+        c->toy_cap = chunk = (std::min(chunk, n_toys) + 1) / 2;
+    }
 }
 
 }  // namespace
@@ -1871,10 +1904,11 @@ int gsn_fit_rates_batch_dev(gsn_ctx* c, int n_toys, double* params_dev, const do
             CUDA_TRY(c, cudaMemsetAsync(c->Mbuf.p, 0, (size_t)T * c->G * S * c->Jmax * sizeof(double), c->stream));
             if ((rc = launch(c, K_COLUMNS, a, launch_columns))) return rc;
             // few toys: the column blocks of the per-species kernel among several CTAs (at most eight waves of
-            // two CTAs per SM), their sums apart in up to 2 GiB; without the memory one CTA adds them as it goes
+            // two CTAs per SM), their sums apart in what the shapes and rows leave of the 4 GiB; without the memory
+            // one CTA adds them as it goes
             const long long ctas = (long long)((c->Jmax + 255) / 256) * c->G * T * ((S + 15) / 16);
             const size_t apart = (size_t)T * c->G * a.nblk * S * c->Jmax * sizeof(double);
-            if (ctas < 16LL * c->nsm && apart <= ((size_t)2 << 30) &&
+            if (ctas < 16LL * c->nsm && apart + T * per_toy <= ((size_t)4 << 30) &&
                 !(c->opt.precision == GSN_FP64 && c->opt.resolution == GSN_RES_GAUSS) &&
                 ensure(c, c->sppart, apart) == GSN_OK) {
                 a.sp_parts = (int)std::min<long long>(a.nblk, (16LL * c->nsm + ctas - 1) / ctas);
