@@ -1189,8 +1189,7 @@ int gsn_create(gsn_ctx** out, const gsn_options* opt) {
     if (c->nsm <= 0) c->nsm = 1;
     if (o.precision == GSN_MIXED && device_ex2_bias(c->dev, c->ex2_bias) != cudaSuccess) {
         cudaGetLastError();
-        if (c->own_stream) cudaStreamDestroy(c->stream);
-        delete c;
+        gsn_destroy(c);
         return GSN_ERR_CUDA;
     }
     *out = c;
