@@ -298,7 +298,7 @@ int pair_tables(gsn_ctx* c, const std::vector<double>& ntab_d, const std::vector
     std::vector<double> tref;
     std::vector<float> snode, qnode;
     std::vector<unsigned char> qn;
-    std::vector<double> gx, gw;   // Gaussian: eight nodes (six-sigma-wide tails of a sigma of half a bin: 1e-16)
+    std::vector<double> gx, gw;   // Gaussian: eight nodes (SQ_GAUSS)
     gauss_legendre(8, gx, gw);
     // the exponent terms of a point x of a tile with reference xr
     auto terms = [&](std::vector<float>& o, double x, double xr) {

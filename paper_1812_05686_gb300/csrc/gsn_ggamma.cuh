@@ -351,21 +351,6 @@ DEV GGSides gg_sides(float p, const float* lam) {
     g.Q2 = gg_q2f(p * g.dlam2, g.E2);
     return g;
 }
-DEV float gg_bin_value_f3(const float* c, float xc, const float* lam, const float* wt, const GGSides& sd) {
-    const float Dx = (xc - c[F_MUH]) - c[F_MUL];
-    float Lc;
-    log1pmx2_f(Dx * c[F_A], Lc);
-    const float p = c[F_KAPPA], Ap = c[F_B], Kp = c[F_C];
-    const float L1 = Lc + lam[1];
-    float e1;
-    const float Q = gg_q2f(p * L1, e1);
-    const float Ql = fmaf(e1, sd.E0, Q + sd.Q0), Qr = fmaf(e1, sd.E2, Q + sd.Q2);
-    const float vl = ex2f(fmaf(-Ap, Ql, Kp * (L1 + sd.dlam0)));
-    const float vc = ex2f(fmaf(-Ap, Q, Kp * L1));
-    const float vr = ex2f(fmaf(-Ap, Qr, Kp * (L1 + sd.dlam2)));
-    return fmaf(wt[0], vl, fmaf(wt[1], vc, wt[2] * vr));
-}
-
 // FP64 bin value: sum_n w_n exp(ln p - d ln s - lnGamma(d/p) + (d-1) ln x_n - (x_n/s)^p)
 template <int NG>
 DEV double gg_bin_value_d(const double* c, const double* lx, const double* wt) {

@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_GGF_MINBLOCKS) k_forward_g
         valid[h] = use[h] && j >= wlo && j < whi;
         const int jr = min(max(j, wlo), max(whi - 1, wlo));
         const int nb = tb_g_node_off(a, g) + min(jr, tb_g_bins(a, g) - 1);
-        if (use[h]) use[h] = !__any_sync(0xffffffffu, a.bclass[nb] != BIN_LIN);  // low tiles: k_forward
+        if (use[h]) use[h] = !__any_sync(0xffffffffu, a.bclass[nb] != BIN_LIN);  // low tiles: k_forward_gg_low
         xlo[h] = INFINITY; xhi[h] = -INFINITY;
         if (use[h]) {
             xlo[h] = (float)a.edges[tb_g_edge_off(a, g) + max(j0, wlo)];

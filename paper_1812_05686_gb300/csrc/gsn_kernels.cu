@@ -447,25 +447,11 @@ DEV int forward_loop(const KArgs& a, int t, int g, int split, float xlo_w, float
     const int kchunk = (a.K + a.nsplit - 1) / a.nsplit;
     const int k_beg = split * kchunk, k_end = min(a.K, k_beg + kchunk);
     const R* blk = reinterpret_cast<const R*>(a.blkbuf) + ((long long)t * a.G + g) * a.nblk * 2;
+    static_assert(sizeof(R) == 8 || RES == 2, "mixed: the free power's low bins only");
+    constexpr int NGM = sizeof(R) == 4 ? NGM_F : NGM_D;
     R del[NG], lam[NG], wt[NG];
-    [[maybe_unused]] GGSides sides{};
-    if constexpr (sizeof(R) == 4) {
 #pragma unroll
-        for (int n = 0; n < NG; ++n) {
-            del[n] = nodes[n]; lam[n] = nodes[NGM_F + n]; wt[n] = valid ? nodes[2 * NGM_F + n] : R(0);
-        }
-        if constexpr (RES == 2 && NG == 3) {
-            // the toy's power (the value every column record of the toy carries)
-            const int q = tb_g_resp(a, g, 5);
-            const float pw = (float)(a.params[(long long)t * a.params_stride + q] * tb_g_rscale(a, g, 5));
-            sides = gg_sides(pw, lam);
-        }
-    } else {
-#pragma unroll
-        for (int n = 0; n < NG; ++n) {
-            del[n] = nodes[n]; lam[n] = nodes[NGM_D + n]; wt[n] = valid ? nodes[2 * NGM_D + n] : R(0);
-        }
-    }
+    for (int n = 0; n < NG; ++n) { del[n] = nodes[n]; lam[n] = nodes[NGM + n]; wt[n] = valid ? nodes[2 * NGM + n] : R(0); }
     for (int b = k_beg / COLBLK + bfirst; b * COLBLK < k_end; b += bstep) {
         if (blk[2 * b + 1] < (R)xlo_w || blk[2 * b] > (R)xhi_w) continue;
         // FP32: partial sums of up to 32 columns folded into compensated (s, cs) pairs
@@ -477,10 +463,8 @@ DEV int forward_loop(const KArgs& a, int t, int g, int split, float xlo_w, float
             ++ncol;
             R v;
             if constexpr (sizeof(R) == 4) {
-                if constexpr (RES == 2 && NG == 3) v = gg_bin_value_f3(c, xc, lam, wt, sides);
-                else if constexpr (RES == 2) v = gg_bin_value_f<NG>(c, xc, lam, wt);
-                else v = bin_value_f<RES, NG>(c, xc, del, lam, wt);
-                if (RES >= 1 && is_zero) v = valid ? zerorec<R>(a, t, g, k)[Z_P0] : 0.0f;
+                v = gg_bin_value_f<NG>(c, xc, lam, wt);
+                if (is_zero) v = valid ? zerorec<R>(a, t, g, k)[Z_P0] : 0.0f;
             } else {
                 if constexpr (RES == 2) v = gg_bin_value_d<NG>(c, lam, wt);
                 else v = bin_value_gamma_d<NG>(c, del, lam, wt);
@@ -517,10 +501,9 @@ DEV void count_work(const KArgs& a, int kind, bool lane_valid, long long n_other
         atomicAdd(&a.work[kind], (unsigned long long)n_other * (unsigned long long)__popc(m));
 }
 
-// lanes <-> bins (32 per warp), loop over the columns of the band.  The FP32 generalized gamma is
-// held to 64 registers: four resident blocks per SM instead of three
-template <class R, int RES>
-__global__ void __launch_bounds__(FWD_WARPS * 32, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_forward(KArgs a) {
+// FP64 gamma family: lanes <-> bins (32 per warp), loop over the columns of the band
+template <int RES>
+__global__ void __launch_bounds__(FWD_WARPS * 32) k_forward(KArgs a) {
     const int tile = blockIdx.x, split = blockIdx.y;
     const int t = blockIdx.z / a.G, g = blockIdx.z % a.G;
     if (!tb_g_active(a, g)) return;  // no smeared species in the group
@@ -540,16 +523,9 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, (sizeof(R) == 4 && RES == 2) ?
     const bool low = __any_sync(0xffffffffu, cls != BIN_LIN);
     double accd[MAXGDS] = {};
     int ncol;
-    if constexpr (sizeof(R) == 4) {
-        const float* nodes = a.ntab_f + (long long)nb * 3 * NGM_F;
-        const float xc = a.xc_f[nb];
-        if (low) ncol = forward_loop<float, RES, NG_LOG_F>(a, t, g, split, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, xc, accd);
-        else     ncol = forward_loop<float, RES, NG_LIN_F>(a, t, g, split, xlo_w, xhi_w, valid, false, nodes, xc, accd);
-    } else {
-        const double* nodes = a.ntab_d + (long long)nb * 3 * NGM_D;
-        if (low) ncol = forward_loop<double, RES, NG_LOG_D>(a, t, g, split, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd);
-        else     ncol = forward_loop<double, RES, NG_LIN_D>(a, t, g, split, xlo_w, xhi_w, valid, false, nodes, 0.0, accd);
-    }
+    const double* nodes = a.ntab_d + (long long)nb * 3 * NGM_D;
+    if (low) ncol = forward_loop<double, RES, NG_LOG_D>(a, t, g, split, xlo_w, xhi_w, valid, cls == BIN_ZERO, nodes, 0.0, accd);
+    else     ncol = forward_loop<double, RES, NG_LIN_D>(a, t, g, split, xlo_w, xhi_w, valid, false, nodes, 0.0, accd);
     count_work(a, K_FORWARD, valid, ncol);
     if (valid) {
         double* out = a.mubuf + ((long long)t * a.nsplit + split) * a.total_bins;
@@ -1027,10 +1003,11 @@ __global__ void __launch_bounds__(256) k_devfinal(KArgs a) {
 }
 
 // ------------------------------------------------------------ backward -----
-// lanes <-> columns; each warp sweeps the bins of its columns' band.  The FP32 generalized gamma is
-// held to 64 registers (four resident blocks per SM instead of three)
+// lanes <-> columns; each warp sweeps the bins of its columns' band: FP64, and the mixed free power with
+// secondary observables, which is held to 64 registers (four resident blocks per SM instead of three)
 template <class R, int RES>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_backward(KArgs a) {
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 1) k_backward(KArgs a) {
+    static_assert(sizeof(R) == 8 || RES == 2, "the other mixed responses: gsn_mixed.cu, gsn_ggmixed.cu");
     const int task = blockIdx.x, g = blockIdx.y, t = blockIdx.z;
     if (!tb_g_active(a, g)) return;  // no smeared species in the group
     const int W = a.bw_warps;
@@ -1193,7 +1170,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_b
                 for (int dd = 0; dd < MAXGDS; ++dd) U0[dd] = fma(wj[dd], rho, U0[dd]);
             }
         }
-    } else if constexpr (sizeof(R) == 8 && RES == 0) {
+    } else if constexpr (RES == 0) {
         // exact Gaussian bin integrals from the edges, derivatives from the edge densities
         const double mu = c[F_MUH], isg = c[F_A];
         double zp = 0, qp = 0, pp = 0;
@@ -1229,49 +1206,11 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_b
             if (secU) Wj += sec_weight(j);
             const unsigned char cls = a.bclass[nbase + j];
             R rho = 0;
-            if (RES == 1 && cls == BIN_ZERO) {
+            if (cls == BIN_ZERO) {
                 const R* zr = zerorec<R>(a, t, g, kval ? k : a.K - 1);
                 rho = zr[Z_P0];
                 U1 = fma(Wj, zr[Z_P0D], U1);
                 U2 = fma(Wj, zr[Z_P0S], U2);
-            } else if constexpr (sizeof(R) == 4) {
-                const float* nd = a.ntab_f + (long long)(nbase + j) * 3 * NGM_F;
-                const float Dx = (a.xc_f[nbase + j] - c[F_MUH]) - c[F_MUL];
-                const int NG = cls == BIN_LOG ? NG_LOG_F : NG_LIN_F;
-                if constexpr (RES == 0) {
-                    const float z = Dx * c[F_A];
-                    float Z1 = 0.f, Z2 = 0.f;
-                    for (int n = 0; n < NG; ++n) {
-                        const float zn = fmaf(nd[n], c[F_A], z);
-                        const float qn = zn * zn;
-                        const float fw = nd[2 * NGM_F + n] * ex2f(-fmaf(0.5f * L2E, qn, qn * HALF_L2E_LO));
-                        rho += fw; Z1 = fmaf(fw, zn, Z1); Z2 = fmaf(fw, fmaf(zn, zn, -1.0f), Z2);
-                    }
-                    U1 = fmaf(Wj, Z1, U1);
-                    U2 = fmaf(Wj, Z2, U2);
-                } else {
-                    // the mixed gamma record (B = d, C = -1/s, KAPPA = ln d - psi(d)): sums of
-                    // (mu/d) d ln f/d mu at fixed variance and s^2 d ln f/d var at fixed mean per node
-                    const float A = c[F_A];
-                    const float tt = Dx * A;
-                    float L1;
-                    const float Dt = log1pmx2_f(tt, L1);
-                    const float P2 = mul_l2e(c[F_B]), Q2 = fmaf(L2E, c[F_B], fmaf(L2E_LO, c[F_B] - 1.0f, -L2E));
-                    const float R2 = mul_l2e(c[F_C]);
-                    const float Ec = fmaf(P2, Dt, fmaf(-L2E, L1, -c[F_XM]));
-                    const float kap = c[F_KAPPA];
-                    float u1 = 0.f, u2 = 0.f;
-                    for (int n = 0; n < NG; ++n) {
-                        const float fw = nd[2 * NGM_F + n] * ex2f(Ec + fmaf(R2, nd[n], Q2 * nd[NGM_F + n]));
-                        const float L1n = L1 + nd[NGM_F + n];
-                        const float tn = fmaf(nd[n], A, tt);
-                        rho += fw;
-                        u1 = fmaf(fw, fmaf(2.0f, L1n + kap, -tn), u1);
-                        u2 = fmaf(fw, -((L1n - tn) + kap), u2);
-                    }
-                    U1 = fmaf(Wj, u1, U1);
-                    U2 = fmaf(Wj, u2, U2);
-                }
             } else {
                 // FP64 gamma: f = exp((d-1) ln x - x/s + A); df/dd = f (ln x - ln s - psi(d)); df/ds = f (x - mu)/s^2
                 const double* nd = a.ntab_d + (long long)(nbase + j) * 3 * NGM_D;
@@ -1311,13 +1250,9 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && RES == 2) ? 4 : 1) k_b
         } else if constexpr (RES == 0) {
             g_mu = U1 * c[F_A];
             g_var = R(0.5) * U2 * c[F_A] * c[F_A];
-        } else if constexpr (sizeof(R) == 4) {
-            g_mu = U1 * (c[F_B] * c[F_A]);     // (d / mu) U1
-            g_var = U2 * (c[F_C] * c[F_C]);    // U2 / s^2
         } else {
-            // fp64: C = 1/s, d = mu / s
-            const R d = sizeof(R) == 4 ? c[F_B] : mu * c[F_C];
-            const R s = sizeof(R) == 4 ? R(-1) / c[F_C] : R(1) / c[F_C];
+            // C = 1/s, d = mu / s
+            const R d = mu * c[F_C], s = R(1) / c[F_C];
             const R var = d * s * s;
             const R gd = U1, gs = U2 * c[F_C] * c[F_C];
             g_mu = gd * (R(2) * d / mu) - gs * (s / mu);
@@ -1395,7 +1330,9 @@ DEV double task_share(const double* row, int nv, int v, int sh, int shares, int 
 
 // Problems of many response groups (GF_GROUPS or more): the partials of every (toy, group) are summed
 // by a block of their own into the group's first task row, and k_gradfinal reads that row only (one
-// block walking 64 groups one after another took 20 us per group)
+// block walking 64 groups one after another took 20 us per group).  One launch / two: 2 groups 26 / 23 us for
+// one toy, 26 / 33 for 512; 4 groups 32 / 25 and 42 / 54; 16 groups 68 / 55 and 146 / 181 (of steps of 0.3 ms for
+// one toy, tens of ms for 512)
 constexpr int GF_GROUPS = 4;
 __global__ void __launch_bounds__(GF_THREADS) k_gradsum(KArgs a) {
     const int t = blockIdx.x, g = blockIdx.y;
@@ -1513,10 +1450,9 @@ DEV void species_loop(const KArgs& a, int t, int g, float xlo_w, float xhi_w, bo
 // grid (bin tiles, groups, toys x species chunks of 16): M[t][g][s][j] (toy stride a.mstride).  Where that
 // leaves the GPU with less than a few waves (a.sp_parts > 0), the column blocks of 256 are dealt in turn to
 // sp_parts CTAs, so that each of a CTA's warps keeps a share of its band; their sums, kept apart in sp_part
-// [t][g][block][s][j], are added in the order in which one CTA adds them: the same bits.  Calls of
-// two-dataset FP64 fits: 64 toys, 512 bins, 20000 columns 78.8 -> 63.6 ms; 10 toys, 1200, 14000 61.0 -> 23.4 ms;
-// 48 toys, 700, 8000, where one CTA per SM fits evenly, 40.2 -> 38.4 ms.  Runs of consecutive blocks instead left
-// most of a CTA's warps without a band to evaluate (73.1, 26.8 and 43.8 ms).
+// [t][g][block][s][j], are added in the order in which one CTA adds them: the same bits.  Two-dataset FP64
+// fits, one CTA -> shared: 64 toys x 512 bins x 20000 columns 78.8 -> 63.6 ms; 10 x 1200 x 14000 61.0 -> 23.4 ms;
+// 48 x 700 x 8000, where one CTA per SM fits evenly, 40.2 -> 38.4 ms.
 template <class R, int RES>
 __global__ void __launch_bounds__(FWD_WARPS * 32) k_species(KArgs a) {
     const int tile = blockIdx.x, g = blockIdx.y;
@@ -1774,7 +1710,9 @@ cudaError_t run_probe(int which, int nsm, double* ops) {
 // ------------------------------------------------------------ launchers ----
 template <class R, int RES, bool FAST>
 static cudaError_t launch_cols(const KArgs& a, cudaStream_t st) {
-    // four blocks of 64 in a cluster where blocks of 256 would leave SMs without work
+    // four blocks of 64 in a cluster where blocks of 256 would leave SMs without work or with a wave or two.
+    // 20000 gamma columns, 256 -> cluster: one toy FP64 87 -> 56, mixed 39 -> 27 us; four 143 -> 105, 41 -> 33; seven
+    // (the line) 182 -> 154, 43 -> 46.  2000 Gaussian columns FP64 24 -> 17 us, one toy or seven
     if ((long long)a.nblk * a.G * a.T < 4LL * a.nsm) {
         cudaLaunchAttribute at[1];
         at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1813,8 +1751,8 @@ cudaError_t launch_forward(const KArgs& a, cudaStream_t st) {
         if (grid.x > 0) k_forward_gg_low<<<grid, FWD_WARPS * 32, 0, st>>>(a);
     } else {
         if (a.res == 0)      k_forward_gauss64<<<grid, FWD_WARPS * 32, 0, st>>>(a);
-        else if (a.res == 1) k_forward<double, 1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
-        else                 k_forward<double, 2><<<grid, FWD_WARPS * 32, 0, st>>>(a);
+        else if (a.res == 1) k_forward<1><<<grid, FWD_WARPS * 32, 0, st>>>(a);
+        else                 k_forward<2><<<grid, FWD_WARPS * 32, 0, st>>>(a);
     }
     return cudaGetLastError();
 }
@@ -1840,9 +1778,7 @@ cudaError_t launch_backward(const KArgs& a, cudaStream_t st) {
     const int threads = a.bw_warps * 32;
     const size_t rs = a.precision == 1 ? sizeof(float) : sizeof(double);
     const size_t sm = rs * MAXGDS * threads + 16 + sizeof(double) * a.bw_warps * NRESP;
-    if (a.precision == 1 && a.res == 0)      k_backward<float, 0><<<grid, threads, sm, st>>>(a);
-    else if (a.precision == 1 && a.res == 1) k_backward<float, 1><<<grid, threads, sm, st>>>(a);
-    else if (a.precision == 1)               k_backward<float, 2><<<grid, threads, sm, st>>>(a);
+    if (a.precision == 1)  k_backward<float, 2><<<grid, threads, sm, st>>>(a);
     else if (a.res == 0)   k_backward<double, 0><<<grid, threads, sm, st>>>(a);
     else if (a.res == 1)   k_backward<double, 1><<<grid, threads, sm, st>>>(a);
     else                   k_backward<double, 2><<<grid, threads, sm, st>>>(a);

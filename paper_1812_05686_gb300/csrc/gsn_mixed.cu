@@ -146,10 +146,10 @@ DEV void share_batches(int sub, int nsub, int& kfirst, int& klast) {
 // node table for all their bins.  They are few (the first one or two of a window) and every column of
 // the lowest ~100 p.e. reaches them, so one warp walking those columns from global memory was the
 // longest chain of a launch: a whole block takes the segment, its warps every eighth batch of 32
-// columns from shared memory, and the warps' sums are added in a fixed order.  With the batches of a
-// split shared among several warps where a launch has few (nsub), the forward of 4 toys x 64 response
-// groups takes 7.8 ms (18.3), of one two-dataset point 66 us (158), of 4096 toys 24.5 ms (28.2: the
-// general path also cost the others registers).
+// columns from shared memory, and the warps' sums are added in a fixed order.  The general path also held
+// registers of every warp.  With the batches of a split shared among several warps where a launch has few
+// (nsub): forward of 4 toys x 64 response groups 18.3 -> 7.8 ms, of one two-dataset point 158 -> 66 us, of
+// 4096 toys 28.2 -> 24.5 ms.
 struct LowRec { float4 r[4]; };
 
 template <int RES, int HALVES>
@@ -554,8 +554,9 @@ __global__ void __launch_bounds__(FWD_WARPS * 32, GSN_FWD_MINBLOCKS) k_forward_m
 // per batch.
 // Groups of three or four datasets keep twice as many accumulators: their adjoint gets the register
 // budget of three resident blocks (80 registers; at 64 it spilled ~300 bytes per thread).  One or two
-// datasets run best with five (48 registers): 4096 toys 34.4 ms with four, 33.7 with five, 38.6 with six;
-// the secondary variant, which needs more, keeps four.
+// datasets run best with five (48 registers).  Four -> five: 4096 gamma toys 34.4 -> 33.7 ms (six: 38.6), 4096
+// Gaussian toys of 900 bins 2.90 -> 2.84 ms, 64 toys of ten groups of one or two datasets 0.86 -> 0.82 and
+// 0.91 -> 0.87 ms; the secondary variant, which needs more, keeps four.
 template <int RES, int NDS, bool FAST, bool SEC>
 __global__ void __launch_bounds__(256, NDS > 2 ? 3 : SEC ? 4 : GSN_BW_MINBLOCKS) k_backward_m(KArgs a) {
     const int task = blockIdx.x, g = blockIdx.y, t = blockIdx.z;

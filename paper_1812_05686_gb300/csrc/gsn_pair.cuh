@@ -8,9 +8,9 @@ namespace gsn {
 constexpr int FM = 16;
 // columns it serves: sigma in bin widths, and the gamma family's shape (d, and mu^2 / sigma^2)
 constexpr double SM_SIGMA = 6.0, SM_SHAPE = 20.0;
-// smallest sigma that the pairs take at all.  Gaussian, in bin widths: the eight nodes of a bin are at
-// 1e-16 of the column there, and at 1e-11 of its value at 8 sigma.  Gamma family, in half widths of a tile of 32 bins: the terms of the exponent are of the
-// size (half width / sigma)^2 / 2 and cancel at the column's peak
+// Smallest sigma that the pairs take at all.  Gaussian, in bin widths: the eight nodes of a bin are off by
+// 5e-20 of the bin at the column's centre, 2e-13 at 8 sigma.  Gamma family, in half widths of a tile of 32
+// bins: the terms of the exponent are of the size (half width / sigma)^2 / 2 and cancel at the column's peak
 constexpr double SQ_GAUSS = 1.5, SQ_GAMMA = 1.0 / 8;
 // weights outside this range (other than 0) keep the FP64 formulas: an FP32 pair would lose its low part
 constexpr double PAIR_TMIN = 1e-25, PAIR_TMAX = 1e30;
@@ -19,9 +19,9 @@ constexpr double SPEC_SCALE = 1152921504606846976.0, SPEC_MIN = 1e-40;
 // a column with more than this share of its batch's weight is evaluated in FP64 beside the pairs
 constexpr float HEAVY_SHARE = 0.25f;
 // Stray bins: counts of 2^20 expectations or more, in the tails where a column's density leaves FP32's range
-// (a tile that a band touches reaches bins 20 sigma out, 1e-87 of the peak) and where w = 1 - n/mu may leave it too.
-// Their expectation and their part of the adjoint take the FP64 formulas.
-// STRAY_RATIO: the same bound on the difference of the high words of n and mu; STRAY_HI: high word of w = -2^20
+// (a tile that a band touches reaches bins 20 sigma out, 1e-87 of the peak) and w = 1 - n/mu may leave it too.
+// Their expectation and their part of the adjoint take the FP64 formulas.  STRAY_RATIO: the bound on the
+// difference of the high words of n and mu; STRAY_HI: high word of w = -2^20
 constexpr int STRAY_RATIO = 20 << 20;
 constexpr unsigned STRAY_HI = 0xC1300000u;
 DEV bool is_stray(double w) { return (unsigned)__double2hiint(w) >= STRAY_HI; }
