@@ -110,7 +110,9 @@ typedef struct gsn_options {
     int    device;         /* CUDA device ordinal */
     void*  stream;         /* cudaStream_t for all work of the context; NULL = a
                               stream created and owned by the context */
-    int    max_toys_per_launch; /* batch chunk bounding scratch memory (<= 0: 4096) */
+    int    max_toys_per_launch; /* batch chunk bounding scratch memory (<= 0: 4096); chunks hold at most
+                              32 GiB of column records, and fewer toys where the device has
+                              less memory left */
     int    use_graphs;     /* 1: gsn_eval_grad and the batch calls record their kernel
                               launches into a CUDA graph on first use and replay it when a
                               call repeats with the same sizes and buffers; 0: plain launches.

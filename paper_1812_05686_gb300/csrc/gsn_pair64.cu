@@ -7,8 +7,8 @@
 // about 55 FP32 operations.  What stays FP64 is done once per 32 pairs (the exponent at a tile's
 // reference point, the flush of the partial sums) and runs on the FP64 pipe beside them.
 // Measured on 128 toys of the two-dataset workload (2 x 1200 bins, 20000 columns): forward 198.7 ->
-// 3.64 ms (103 instructions per 32 pairs, issue 72%, FMA pipe 52%, FP64 pipe 43%), adjoint 186.3 -> 6.37 ms
-// (164 instructions), per-species shapes of one point 72 -> 0.21 ms; 500 toys of the 900-bin Gaussian
+// 3.62 ms (103 instructions per 32 pairs, issue 73%, FMA pipe 54%, FP64 pipe 44%), adjoint 186.3 -> 6.37 ms
+// (165 instructions), per-species shapes of one point 72 -> 0.21 ms; 500 toys of the 900-bin Gaussian
 // workload: forward 44.6 -> 0.86 ms, adjoint 49.5 -> 1.17 ms.  Errors against 64-bit references, before
 // -> now: gradients of the gamma toys 3.4e-13 -> 3.2e-13, of the Gaussian toys 8.9e-15 -> 8.6e-15.
 //
